@@ -10,8 +10,6 @@
 namespace tq {
 cudaError_t launch_rowptr(int N, int K, const uint32_t *sal, int32_t *rowptr, uint32_t *status,
                           cudaStream_t s);
-cudaError_t launch_check_rowptr(int N, int K, const uint32_t *sal, const int32_t *rowptr,
-                                uint32_t *status, cudaStream_t s);
 cudaError_t launch_pack(int N, int K, const int8_t *T1, const int8_t *T2, const uint32_t *sal,
                         const int32_t *rowptr, uint8_t *plane1, uint8_t *plane2, uint32_t *status,
                         cudaStream_t s);
@@ -241,9 +239,7 @@ tq_status tq_pack(int32_t N, int32_t K, const int8_t *T1, const int8_t *T2, cons
   if (tq_status st = check_shape(N, K)) return st;
   if (!T1 || !sal || !rowptr || !plane1 || !d_status) return TQ_ERR_NULL;
   if ((T2 == nullptr) != (plane2 == nullptr)) return TQ_ERR_NULL;
-  cudaStream_t s = (cudaStream_t)stream;
-  if (tq_status st = from_cuda(launch_check_rowptr(N, K, sal, rowptr, d_status, s))) return st;
-  return from_cuda(launch_pack(N, K, T1, T2, sal, rowptr, plane1, plane2, d_status, s));
+  return from_cuda(launch_pack(N, K, T1, T2, sal, rowptr, plane1, plane2, d_status, (cudaStream_t)stream));
 }
 
 tq_status tq_unpack(int32_t N, int32_t K, const uint8_t *plane1, const uint8_t *plane2,
@@ -251,9 +247,7 @@ tq_status tq_unpack(int32_t N, int32_t K, const uint8_t *plane1, const uint8_t *
                     uint32_t *d_status, void *stream) {
   if (tq_status st = check_shape(N, K)) return st;
   if (!plane1 || !sal || !rowptr || !T1 || !d_status) return TQ_ERR_NULL;
-  cudaStream_t s = (cudaStream_t)stream;
-  if (tq_status st = from_cuda(launch_check_rowptr(N, K, sal, rowptr, d_status, s))) return st;
-  return from_cuda(launch_unpack(N, K, plane1, plane2, sal, rowptr, T1, T2, d_status, s));
+  return from_cuda(launch_unpack(N, K, plane1, plane2, sal, rowptr, T1, T2, d_status, (cudaStream_t)stream));
 }
 
 size_t tq_plane2_index_capacity(int32_t K, int64_t nnz) {

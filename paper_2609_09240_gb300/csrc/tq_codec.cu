@@ -216,143 +216,286 @@ __global__ void unpack_kernel(int N, int K, const uint8_t *plane1, const uint8_t
   }
 }
 
-// ------------------------------------------------ row-staged pack / unpack
-// The same byte layout and status bits as pack_kernel / unpack_kernel, with
-// one CTA per row at a time.  The row's codes move between global and
-// shared memory in 16-byte units (coalesced), and the per-byte encode or
-// decode works on shared memory; the salience rank of each group is formed
-// once per row.  Taken when the code arrays are 16-byte aligned and a row's
-// codes fit in shared memory.
-constexpr int kPackThreads = 128;    // pack: up to 16 CTAs (rows in flight) per SM
-constexpr int kUnpackThreads = 256;
-constexpr int kRowMaxK = 49152;  // 2 x 48 KiB of codes per row
+// ----------------------------------------------- warp-staged pack / unpack
+// The same bytes and status bits as pack_kernel / unpack_kernel, a warp per
+// 32 consecutive groups (of one row or several).  The codes move between
+// global and shared memory in 16-byte units (a warp's 4 KB are contiguous),
+// each lane encodes or decodes one group in registers, and the packed bytes
+// move in 2-byte units, 64 contiguous bytes per access.  Taken when the code
+// arrays are 16-byte and the packed planes 2-byte aligned.
+// What bounds it: HBM (the codes, read or written once).  A warp has its 8 KB
+// of codes under way at once and waits for no other warp; with a CTA per row
+// and block barriers between load, encode and store, packing and unpacking a
+// 12288 x 4096 projection took 120 us (1.87 TB/s), this takes 58 us (3.87 TB/s;
+// pack 33, unpack 30 of them under a profiler, at about 45 % issue).
+constexpr int kCodecWarps = 4;
+constexpr int kGroupStride = kGroup + 16;  // a group's codes in shared memory (free of bank conflicts)
+constexpr int kStageBytesW = 32 * kGroupStride;
 
-// The byte of the five codes row[k0 .. k0 + 4] (a full byte): two 32-bit
-// shared-memory loads and a funnel shift give the codes, their digits
-// (code + 1) come bytewise without carries between bytes, and one dp4a
-// forms sum d_i 3^i.  A code outside {-1, 0, 1} goes through encode_codes,
-// which clamps it and flags the status.
-__device__ __forceinline__ uint8_t encode5(const int8_t *row, int k0, uint32_t *st) {
-  const uint32_t *w = reinterpret_cast<const uint32_t *>(row) + (k0 >> 2);
-  const uint32_t sh = 8u * (uint32_t)(k0 & 3);
-  const uint32_t lo = w[0], hi = w[1];
-  const uint32_t c4 = __funnelshift_r(lo, hi, sh), c5 = (hi >> sh) & 0xFFu;
-  const uint32_t d4 = ((c4 & 0x7F7F7F7Fu) + 0x01010101u) ^ (c4 & 0x80808080u);
-  const uint32_t d5 = ((c5 & 0x7Fu) + 1u) ^ (c5 & 0x80u);
-  if ((((d4 | d5) & 0xFCFCFCFCu) | (d4 & (d4 >> 1) & 0x01010101u) | (d5 & (d5 >> 1) & 1u)) != 0)
-    return encode_codes(row + k0, 5, st);
-  return (uint8_t)__dp4a(d4, 0x1B090301u, 81u * d5);
+// Digits (code + 1) of four codes, bytewise without carries between bytes.
+__device__ __forceinline__ uint32_t digits4(uint32_t c) {
+  return ((c & 0x7F7F7F7Fu) + 0x01010101u) ^ (c & 0x80808080u);
+}
+// Bits that are set iff some digit is not 0, 1 or 2.
+__device__ __forceinline__ uint32_t not_digits4(uint32_t d) { return (d & 0xFCFCFCFCu) | (d & (d >> 1) & 0x01010101u); }
+
+// The 26 bytes of a group from its 128 codes in shared memory (p), as
+// halfwords; a group with an invalid code goes through encode_codes.
+__device__ __forceinline__ void encode_group(const unsigned char *p, uint16_t (&h)[13], uint32_t *st) {
+  uint32_t d[32], bad = 0;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const uint4 v = *reinterpret_cast<const uint4 *>(p + 16 * i);
+    d[4 * i] = digits4(v.x), d[4 * i + 1] = digits4(v.y), d[4 * i + 2] = digits4(v.z), d[4 * i + 3] = digits4(v.w);
+  }
+#pragma unroll
+  for (int i = 0; i < 32; ++i) bad |= not_digits4(d[i]);
+  if (bad) {
+#pragma unroll 1
+    for (int j = 0; j < 13; ++j) {
+      const int8_t *t = reinterpret_cast<const int8_t *>(p) + 10 * j;
+      const uint32_t lo = encode_codes(t, 5, st), hi = encode_codes(t + 5, j < 12 ? 5 : kTailTrits, st);
+#pragma unroll
+      for (int k = 0; k < 13; ++k)  // (no dynamic register index)
+        if (k == j) h[k] = (uint16_t)(lo | hi << 8);
+    }
+    return;
+  }
+  // byte j: digits 5 j .. 5 j + 4, from the two or three words they lie in
+  auto byte = [&](int j) -> uint32_t {
+    constexpr uint32_t pw[5] = {1, 3, 9, 27, 81};
+    uint32_t v = j < kFullBytes ? 0u : 27u + 81u;  // the tail byte's pad digits are 1
+#pragma unroll
+    for (int w = 5 * j / 4; w <= (5 * j + 4) / 4 && w < 32; ++w) {
+      uint32_t wt = 0;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const int i = 4 * w + k - 5 * j;
+        if (i >= 0 && i < 5) wt |= pw[i] << (8 * k);
+      }
+      v = __dp4a(d[w], wt, v);
+    }
+    return v;
+  };
+#pragma unroll
+  for (int j = 0; j < 13; ++j) h[j] = (uint16_t)(byte(2 * j) | byte(2 * j + 1) << 8);
 }
 
-__host__ __device__ inline int rows_smem_bytes(int K) { return 2 * K + 4 * (K / kGroup); }
-
-// rk[g]: rank of group g among row n's salient groups, -1 if not salient.
-__device__ __forceinline__ void row_ranks(const uint32_t *sal, int W, int G, int n, int32_t *rk) {
-  for (int g = threadIdx.x; g < G; g += blockDim.x) rk[g] = sal_bit(sal, W, n, g) ? sal_rank(sal, W, n, g) : -1;
+// A lane's group of a warp's 32: row, group in the row, whether it exists.
+struct LaneGroup {
+  int n, g;
+  bool live;
+};
+__device__ __forceinline__ LaneGroup lane_group(int64_t q0, int64_t total, int G, int lane) {
+  LaneGroup r;
+  const int64_t n0 = q0 / G;
+  const int e = (int)(q0 - n0 * G) + lane;
+  r.n = (int)n0 + e / G;
+  r.g = e % G;
+  r.live = q0 + lane < total;
+  return r;
+}
+// Halfword u of the warp's packed bytes: lane u / 13's group, its byte
+// 2 (u % 13); off: a lane's byte offset in plane 1, or -1 for no group.
+// (13 accesses of 64 contiguous bytes.)
+template <class F>
+__device__ __forceinline__ void for_halfwords(int64_t off, int lane, F f) {
+#pragma unroll
+  for (int i = 0; i < 13; ++i) {
+    const int u = 32 * i + lane, l = u / 13;
+    const int64_t o = __shfl_sync(0xffffffffu, off, l);
+    f(u, o < 0 ? o : o + 2 * (u - 13 * l));
+  }
+}
+// The check of a row's salience bits and row pointers (check_rowptr_kernel).
+__device__ __forceinline__ uint32_t row_status(const uint32_t *sal, const int32_t *rowptr, int W, int G, int n) {
+  bool pad_bad = false;
+  const int c = row_popc(sal, W, G, n, &pad_bad);
+  uint32_t st = pad_bad ? TQ_DATA_BAD_PAD : 0u;
+  if (rowptr[n + 1] - rowptr[n] != c || (n == 0 && rowptr[0] != 0)) st |= TQ_DATA_BAD_ROWPTR;
+  return st;
 }
 
-__global__ void __launch_bounds__(kPackThreads) pack_rows_kernel(int N, int K, const int8_t *T1, const int8_t *T2,
-                                                               const uint32_t *sal, const int32_t *rowptr,
-                                                               uint8_t *plane1, uint8_t *plane2, uint32_t *status) {
-  extern __shared__ __align__(16) unsigned char smr[];
-  const int G = K / kGroup, W = sal_words_of(K);
-  const int RB = (int)row_bytes_of(K);
-  const int32_t nnz = rowptr[N];
-  int8_t *t1 = reinterpret_cast<int8_t *>(smr), *t2 = t1 + K;
-  int32_t *rk = reinterpret_cast<int32_t *>(smr + 2 * K);
-  uint32_t st = 0;
-  for (int n = blockIdx.x; n < N; n += gridDim.x) {
-    __syncthreads();  // the previous row's shared-memory reads are done
-    row_ranks(sal, W, G, n, rk);
-    const int4 *s1 = reinterpret_cast<const int4 *>(T1 + (int64_t)n * K);
-    for (int i = threadIdx.x; i < K / 16; i += blockDim.x) reinterpret_cast<int4 *>(t1)[i] = __ldcs(s1 + i);
-    if (T2) {
-      const int4 *s2 = reinterpret_cast<const int4 *>(T2 + (int64_t)n * K);
-      for (int i = threadIdx.x; i < K / 16; i += blockDim.x) {
-        const int4 v = __ldcs(s2 + i);
-        reinterpret_cast<int4 *>(t2)[i] = v;
-        // second-plane codes outside the salient groups must be zero
-        if ((v.x | v.y | v.z | v.w) != 0 && !sal_bit(sal, W, n, (16 * i) / kGroup)) st |= TQ_DATA_T2_OUTSIDE;
+__global__ void __launch_bounds__(32 * kCodecWarps) pack_warp_kernel(int N, int K, const int8_t *T1, const int8_t *T2,
+                                                                   const uint32_t *sal, const int32_t *rowptr,
+                                                                   uint8_t *plane1, uint8_t *plane2,
+                                                                   uint32_t *status) {
+  __shared__ __align__(16) unsigned char stage[kCodecWarps][kStageBytesW];
+  const int G = K / kGroup, W = sal_words_of(K), lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t RB = row_bytes_of(K), total = (int64_t)N * G;
+  const int64_t q0 = ((int64_t)blockIdx.x * kCodecWarps + warp) * 32;
+  if (q0 >= total) return;
+  unsigned char *sm = stage[warp];
+  // chunk 32 i + lane of the warp's codes: group 4 i + lane / 8's 16-byte part lane % 8
+  const int64_t chunks = (total - q0) * 8;
+  const uint4 *s1 = reinterpret_cast<const uint4 *>(T1 + q0 * kGroup), *s2 = reinterpret_cast<const uint4 *>(T2 + q0 * kGroup);
+  const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+  uint4 v1[8], v2[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) v1[i] = 32 * i + lane < chunks ? __ldcs(s1 + 32 * i + lane) : zero;
+  if (T2) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v2[i] = 32 * i + lane < chunks ? __ldcs(s2 + 32 * i + lane) : zero;
+  }
+  const LaneGroup L = lane_group(q0, total, G, lane);
+  const int64_t off = L.live ? L.n * RB + (int64_t)L.g * kGroupBytes : -1;
+  const bool s = L.live && sal_bit(sal, W, L.n, L.g);
+  const uint32_t smask = __ballot_sync(0xffffffffu, s);
+  uint32_t st = L.live && L.g == 0 ? row_status(sal, rowptr, W, G, L.n) : 0u;
+  unsigned char *mine = sm + lane * kGroupStride;
+  unsigned char *part = sm + (lane >> 3) * kGroupStride + 16 * (lane & 7);
+  uint16_t h[13];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) *reinterpret_cast<uint4 *>(part + 4 * i * kGroupStride) = v1[i];
+  __syncwarp();
+  encode_group(mine, h, &st);
+  __syncwarp();
+  // the bytes go out in order: through shared memory
+#pragma unroll
+  for (int j = 0; j < 13; ++j) *reinterpret_cast<uint16_t *>(sm + lane * kGroupBytes + 2 * j) = h[j];
+  __syncwarp();
+  for_halfwords(off, lane, [&](int u, int64_t o) {
+    if (o >= 0) *reinterpret_cast<uint16_t *>(plane1 + o) = *reinterpret_cast<const uint16_t *>(sm + 2 * u);
+  });
+  if (L.live && L.g == G - 1)
+    for (int64_t b = off + kGroupBytes; b < (L.n + 1) * RB; b += 2) *reinterpret_cast<uint16_t *>(plane1 + b) = 0;
+  if (T2) {
+    __syncwarp();
+    // second-plane codes outside the salient groups must be zero; the salient
+    // groups' go through shared memory
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const bool sg = (smask >> (4 * i + (lane >> 3))) & 1u;
+      if (sg)
+        *reinterpret_cast<uint4 *>(part + 4 * i * kGroupStride) = v2[i];
+      else if ((v2[i].x | v2[i].y | v2[i].z | v2[i].w) != 0)
+        st |= TQ_DATA_T2_OUTSIDE;
+    }
+    __syncwarp();
+    if (s) {
+      encode_group(mine, h, &st);
+      const int64_t j = (int64_t)rowptr[L.n] + sal_rank(sal, W, L.n, L.g);
+      if (j >= 0 && j < rowptr[N]) {
+        uint16_t *d = reinterpret_cast<uint16_t *>(plane2 + j * kGroupBytes);
+#pragma unroll
+        for (int k = 0; k < 13; ++k) d[k] = h[k];
+      } else {
+        st |= TQ_DATA_BAD_ROWPTR;
       }
     }
-    __syncthreads();
-    const int64_t p1 = (int64_t)n * RB;
-    const int32_t rp = rowptr[n];
-    for (int b = threadIdx.x; b < RB; b += blockDim.x) {
-      if (b >= G * kGroupBytes) {
-        plane1[p1 + b] = 0;
-        continue;
-      }
-      const int g = b / kGroupBytes, pos = b - g * kGroupBytes;
-      const int ntr = pos < kFullBytes ? 5 : kTailTrits;
-      const int k0 = g * kGroup + 5 * pos;
-      plane1[p1 + b] = ntr == 5 ? encode5(t1, k0, &st) : encode_codes(t1 + k0, ntr, &st);
-      const int r = rk[g];
-      if (r >= 0) {
-        if (T2) {
-          const int64_t j = (int64_t)rp + r;
-          if (j >= 0 && j < nnz)
-            plane2[j * kGroupBytes + pos] = ntr == 5 ? encode5(t2, k0, &st) : encode_codes(t2 + k0, ntr, &st);
-          else
-            st |= TQ_DATA_BAD_ROWPTR;
+  } else if (s) {
+    st |= TQ_DATA_T2_OUTSIDE;
+  }
+  st = __reduce_or_sync(0xffffffffu, st);
+  if (st && lane == 0) atomicOr(status, st);
+}
+
+// Decode table: a byte's five codes in bytes 0..4, byte 5 nonzero for an
+// invalid byte (its codes are zero).
+__device__ __forceinline__ uint2 decode_entry(int v) {
+  if (v > 242) return make_uint2(0u, 0x100u);
+  uint32_t t[5];
+#pragma unroll
+  for (int i = 0; i < 5; ++i, v /= 3) t[i] = (uint32_t)(v % 3 - 1) & 0xFFu;
+  return make_uint2(t[0] | t[1] << 8 | t[2] << 16 | t[3] << 24, t[4]);
+}
+// A group's 128 codes into shared memory (p) from its 26 bytes (halfwords).
+__device__ __forceinline__ void decode_group_codes(const uint16_t (&h)[13], const uint2 *lut, unsigned char *p, uint32_t *st) {
+  uint32_t bad = 0, w[32];
+  uint2 e = lut[h[0] & 0xFFu];
+#pragma unroll
+  for (int j = 0; j < 26; ++j) {
+    bad |= e.y;
+    const uint2 nx = j + 1 < 26 ? lut[(j & 1) ? h[(j + 1) >> 1] & 0xFFu : h[j >> 1] >> 8] : make_uint2(0u, 0u);
+    // words whose first code is in byte j: code 4 k = 5 j + i
+#pragma unroll
+    for (int k = (5 * j + 3) / 4; 4 * k < 5 * j + 5 && k < 32; ++k) {
+      const int i = 4 * k - 5 * j;
+      const uint32_t tail = __byte_perm(e.y, nx.x, 0x6540);  // code 4, the next byte's codes 0..2
+      w[k] = i == 0 ? e.x : i == 4 ? tail : __funnelshift_r(e.x, tail, 8 * i);
+    }
+    if (j == 25 && !(e.y & 0x100u) && ((e.x >> 24) | (e.y & 0xFFu))) *st |= TQ_DATA_BAD_PAD;
+    e = nx;
+  }
+  if (bad & 0x100u) *st |= TQ_DATA_BAD_BYTE;
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+    *reinterpret_cast<uint4 *>(p + 16 * i) = make_uint4(w[4 * i], w[4 * i + 1], w[4 * i + 2], w[4 * i + 3]);
+}
+
+__global__ void __launch_bounds__(32 * kCodecWarps) unpack_warp_kernel(int N, int K, const uint8_t *plane1,
+                                                                     const uint8_t *plane2, const uint32_t *sal,
+                                                                     const int32_t *rowptr, int8_t *T1, int8_t *T2,
+                                                                     uint32_t *status) {
+  __shared__ __align__(16) unsigned char stage[kCodecWarps][kStageBytesW];
+  __shared__ __align__(16) uint2 lut[256];
+  const int G = K / kGroup, W = sal_words_of(K), lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t RB = row_bytes_of(K), total = (int64_t)N * G;
+  const int64_t q0 = ((int64_t)blockIdx.x * kCodecWarps + warp) * 32;
+  for (int v = threadIdx.x; v < 256; v += 32 * kCodecWarps) lut[v] = decode_entry(v);
+  unsigned char *sm = stage[warp];
+  const LaneGroup L = lane_group(q0, total, G, lane);
+  const int64_t off = L.live ? L.n * RB + (int64_t)L.g * kGroupBytes : -1;
+  uint16_t x[13];
+  for_halfwords(off, lane, [&](int u, int64_t o) {
+    x[u >> 5] = o >= 0 ? __ldcs(reinterpret_cast<const unsigned short *>(plane1 + o)) : (unsigned short)0;
+  });
+  const bool s = L.live && sal_bit(sal, W, L.n, L.g);
+  const uint32_t smask = __ballot_sync(0xffffffffu, s);
+  uint32_t st = L.live && L.g == 0 ? row_status(sal, rowptr, W, G, L.n) : 0u;
+  if (L.live && L.g == G - 1)
+    for (int64_t b = off + kGroupBytes; b < (L.n + 1) * RB; ++b)
+      if (plane1[b] != 0) st |= TQ_DATA_BAD_PAD;
+  __syncthreads();  // the table
+  if (q0 >= total) return;
+#pragma unroll
+  for (int i = 0; i < 13; ++i) *reinterpret_cast<uint16_t *>(sm + 2 * (32 * i + lane)) = x[i];
+  __syncwarp();
+  uint16_t h[13];
+#pragma unroll
+  for (int j = 0; j < 13; ++j) h[j] = *reinterpret_cast<const uint16_t *>(sm + lane * kGroupBytes + 2 * j);
+  __syncwarp();
+  unsigned char *mine = sm + lane * kGroupStride;
+  const unsigned char *part = sm + (lane >> 3) * kGroupStride + 16 * (lane & 7);
+  uint32_t sd = 0;
+  decode_group_codes(h, lut, mine, &sd);
+  if (L.live) st |= sd;
+  __syncwarp();
+  const int64_t chunks = (total - q0) * 8;
+  uint4 *d1 = reinterpret_cast<uint4 *>(T1 + q0 * kGroup), *d2 = reinterpret_cast<uint4 *>(T2 + q0 * kGroup);
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+    if (32 * i + lane < chunks) __stcs(d1 + 32 * i + lane, *reinterpret_cast<const uint4 *>(part + 4 * i * kGroupStride));
+  if (T2) {
+    // salient groups' records through shared memory, zeros elsewhere
+    // (a record per lane; a byte per lane, record after record, took 5 us more)
+    if (smask) {
+      __syncwarp();
+      if (s) {
+        const int64_t j = (int64_t)rowptr[L.n] + sal_rank(sal, W, L.n, L.g);
+        if (plane2 && j >= 0 && j < rowptr[N]) {
+          const uint16_t *r = reinterpret_cast<const uint16_t *>(plane2 + j * kGroupBytes);
+#pragma unroll
+          for (int k = 0; k < 13; ++k) h[k] = __ldcs(r + k);
+          decode_group_codes(h, lut, mine, &st);
         } else {
-          st |= TQ_DATA_T2_OUTSIDE;
+          st |= TQ_DATA_BAD_ROWPTR;
+#pragma unroll
+          for (int i = 0; i < 8; ++i) *reinterpret_cast<uint4 *>(mine + 16 * i) = make_uint4(0u, 0u, 0u, 0u);
         }
       }
+      __syncwarp();
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const bool sg = (smask >> (4 * i + (lane >> 3))) & 1u;
+      if (32 * i + lane < chunks)
+        __stcs(d2 + 32 * i + lane,
+               sg ? *reinterpret_cast<const uint4 *>(part + 4 * i * kGroupStride) : make_uint4(0u, 0u, 0u, 0u));
     }
   }
-  if (st) atomicOr(status, st);
-}
-
-__global__ void __launch_bounds__(kUnpackThreads) unpack_rows_kernel(int N, int K, const uint8_t *plane1,
-                                                                 const uint8_t *plane2, const uint32_t *sal,
-                                                                 const int32_t *rowptr, int8_t *T1, int8_t *T2,
-                                                                 uint32_t *status) {
-  extern __shared__ __align__(16) unsigned char smr[];
-  const int G = K / kGroup, W = sal_words_of(K);
-  const int RB = (int)row_bytes_of(K);
-  const int32_t nnz = rowptr[N];
-  int8_t *t1 = reinterpret_cast<int8_t *>(smr), *t2 = t1 + K;
-  int32_t *rk = reinterpret_cast<int32_t *>(smr + 2 * K);
-  uint32_t st = 0;
-  for (int n = blockIdx.x; n < N; n += gridDim.x) {
-    __syncthreads();  // the previous row's stores have read shared memory
-    row_ranks(sal, W, G, n, rk);
-    // second-plane codes are zero outside the salient groups: the row starts
-    // zeroed by 16-byte stores, and only salient groups are decoded into it
-    if (T2)
-      for (int i = threadIdx.x; i < K / 16; i += blockDim.x) reinterpret_cast<int4 *>(t2)[i] = make_int4(0, 0, 0, 0);
-    __syncthreads();
-    const int64_t p1 = (int64_t)n * RB;
-    const int32_t rp = rowptr[n];
-    for (int b = threadIdx.x; b < RB; b += blockDim.x) {
-      const uint8_t v = __ldcs(plane1 + p1 + b);
-      if (b >= G * kGroupBytes) {
-        if (v != 0) st |= TQ_DATA_BAD_PAD;
-        continue;
-      }
-      const int g = b / kGroupBytes, pos = b - g * kGroupBytes;
-      const int ntr = pos < kFullBytes ? 5 : kTailTrits;
-      const int k0 = g * kGroup + 5 * pos;
-      decode_to(v, ntr, t1 + k0, &st);
-      if (T2) {
-        const int r = rk[g];
-        const int64_t j = (int64_t)rp + r;
-        if (r >= 0 && plane2 && j >= 0 && j < nnz)
-          decode_to(plane2[j * kGroupBytes + pos], ntr, t2 + k0, &st);
-        else if (r >= 0)
-          st |= TQ_DATA_BAD_ROWPTR;
-      }
-    }
-    __syncthreads();
-    int4 *d1 = reinterpret_cast<int4 *>(T1 + (int64_t)n * K);
-    for (int i = threadIdx.x; i < K / 16; i += blockDim.x) __stcs(d1 + i, reinterpret_cast<const int4 *>(t1)[i]);
-    if (T2) {
-      int4 *d2 = reinterpret_cast<int4 *>(T2 + (int64_t)n * K);
-      for (int i = threadIdx.x; i < K / 16; i += blockDim.x) __stcs(d2 + i, reinterpret_cast<const int4 *>(t2)[i]);
-    }
-  }
-  if (st) atomicOr(status, st);
+  st = __reduce_or_sync(0xffffffffu, st);
+  if (st && lane == 0) atomicOr(status, st);
 }
 
 // ------------------------------------------------------ second-plane index
@@ -521,19 +664,27 @@ cudaError_t launch_check_rowptr(int N, int K, const uint32_t *sal, const int32_t
   return cudaGetLastError();
 }
 
+// Whether the warp-staged kernels take these arrays.
+static bool warp_codec(int N, int K, const void *T1, const void *T2, const void *plane1, const void *plane2) {
+  const int64_t warps = ((int64_t)N * (K / kGroup) + 31) / 32;
+  return ((((uintptr_t)T1) | ((uintptr_t)T2)) & 15u) == 0 && ((((uintptr_t)plane1) | ((uintptr_t)plane2)) & 1u) == 0 &&
+         (warps + kCodecWarps - 1) / kCodecWarps <= INT32_MAX;
+}
+static unsigned warp_codec_blocks(int N, int K) {
+  return (unsigned)(((int64_t)N * (K / kGroup) + 32 * kCodecWarps - 1) / (32 * kCodecWarps));
+}
+
+// Both check the salience map against rowptr as they go (per row; the
+// per-byte kernels by a kernel of its own in front).
 cudaError_t launch_pack(int N, int K, const int8_t *T1, const int8_t *T2, const uint32_t *sal,
                         const int32_t *rowptr, uint8_t *plane1, uint8_t *plane2, uint32_t *status,
                         cudaStream_t s) {
-  if (K <= kRowMaxK && ((((uintptr_t)T1) | ((uintptr_t)T2)) & 15u) == 0) {
-    const int sm = rows_smem_bytes(K);
-    if (sm > 48 * 1024) {
-      const cudaError_t e = cudaFuncSetAttribute(pack_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-      if (e != cudaSuccess) return e;
-    }
-    pack_rows_kernel<<<std::min(N, 152 * 16), kPackThreads, sm, s>>>(N, K, T1, T2, sal, rowptr, plane1, plane2,
-                                                                    status);
+  if (warp_codec(N, K, T1, T2, plane1, plane2)) {
+    pack_warp_kernel<<<warp_codec_blocks(N, K), 32 * kCodecWarps, 0, s>>>(N, K, T1, T2, sal, rowptr, plane1, plane2,
+                                                                         status);
     return cudaGetLastError();
   }
+  if (cudaError_t e = launch_check_rowptr(N, K, sal, rowptr, status, s)) return e;
   pack_kernel<<<std::min(N, 152 * 16), 256, 0, s>>>(N, K, T1, T2, sal, rowptr, plane1, plane2, status);
   return cudaGetLastError();
 }
@@ -541,16 +692,12 @@ cudaError_t launch_pack(int N, int K, const int8_t *T1, const int8_t *T2, const 
 cudaError_t launch_unpack(int N, int K, const uint8_t *plane1, const uint8_t *plane2,
                           const uint32_t *sal, const int32_t *rowptr, int8_t *T1, int8_t *T2,
                           uint32_t *status, cudaStream_t s) {
-  if (K <= kRowMaxK && ((((uintptr_t)T1) | ((uintptr_t)T2)) & 15u) == 0) {
-    const int sm = rows_smem_bytes(K);
-    if (sm > 48 * 1024) {
-      const cudaError_t e = cudaFuncSetAttribute(unpack_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-      if (e != cudaSuccess) return e;
-    }
-    unpack_rows_kernel<<<std::min(N, 152 * 8), kUnpackThreads, sm, s>>>(N, K, plane1, plane2, sal, rowptr, T1, T2,
-                                                                      status);
+  if (warp_codec(N, K, T1, T2, plane1, plane2)) {
+    unpack_warp_kernel<<<warp_codec_blocks(N, K), 32 * kCodecWarps, 0, s>>>(N, K, plane1, plane2, sal, rowptr, T1, T2,
+                                                                           status);
     return cudaGetLastError();
   }
+  if (cudaError_t e = launch_check_rowptr(N, K, sal, rowptr, status, s)) return e;
   unpack_kernel<<<std::min(N, 152 * 16), 256, 0, s>>>(N, K, plane1, plane2, sal, rowptr, T1, T2,
                                                      status);
   return cudaGetLastError();

@@ -206,3 +206,50 @@ def test_plane2_index_bit_exact(H, N, K, frac):
     got = idx.view(np.uint8)[so:].reshape(cap, 32)
     bad = np.nonzero((got != slots).any(axis=1))[0]
     assert bad.size == 0, f"{bad.size} slots differ; first {bad[0]}: {got[bad[0]]} vs {slots[bad[0]]}"
+
+
+@pytest.mark.parametrize("N,K,offset", [(1, 128, 0), (31, 128, 0), (33, 128, 0), (129, 128, 0), (5, 896, 0), (41, 1408, 0),
+                                        (3, 4224, 0), (2, 49280, 0), (16, 4096, 1)])
+def test_pack_unpack_warp_tiles(H, N, K, offset):
+    """Warps of the packing kernels take 32 consecutive groups: fewer than
+    that in all, rows that end inside a warp (with their pad bytes), one group
+    per row, many rows per warp, and packed planes that are not 2-byte aligned
+    (which the per-byte kernels take).  Planted invalid codes, second-plane
+    codes outside the salient groups and invalid bytes, in the first and last
+    group, set the oracle's status bits and give its bytes."""
+    from paper_2609_09240_gb300 import tq
+    w = wl.gen_weights(N, K, 0.3, config=7, proj=5 * N + K)
+    rp, st = oracle.rowptr(N, K, w.sal)
+    assert st == 0
+    nnz = int(rp[-1])
+
+    def buf(n):
+        return torch.full((n + offset,), 9, dtype=torch.uint8, device="cuda")[offset:]
+
+    for plant in (False, True):
+        T1, T2 = w.T1.copy(), w.T2.copy()
+        if plant:
+            T1[0, 3], T1[-1, K - 1] = 2, -3
+            out = np.argwhere(~w.sal_dense)
+            if len(out):
+                T2[out[-1][0], out[-1][1] * 128 + 127] = 1
+        p1_o, p2_o, st_o = oracle.pack(N, K, T1, T2, w.sal, rp)
+        rb = tq.tq_row_bytes(K)
+        p1, p2 = buf(N * rb), buf(max(nnz, 1) * 26)
+        status = torch.zeros(1, dtype=torch.int32, device="cuda")
+        sal, rowptr = H.dev(w.sal), H.dev(rp)
+        tq.tq_pack(N, K, H.dev(T1), H.dev(T2), sal, rowptr, p1, p2, status)
+        assert int(status.item()) == st_o
+        assert np.array_equal(p1.cpu().numpy().reshape(N, rb), p1_o)
+        assert nnz == 0 or np.array_equal(p2.cpu().numpy()[:26 * nnz].reshape(-1, 26), p2_o[:nnz])
+        if plant:
+            p1[0] = 250
+            p1[(N - 1) * rb + K // 128 * 26 - 1] = 0  # tail byte: pad digits 0
+        b1 = p1.cpu().numpy().reshape(N, rb)
+        T1_o, T2_o, st_o = oracle.unpack(N, K, b1, p2_o, w.sal, rp)
+        status.zero_()
+        U1 = torch.full((N, K), 7, dtype=torch.int8, device="cuda")
+        U2 = torch.full((N, K), 7, dtype=torch.int8, device="cuda")
+        tq.tq_unpack(N, K, p1, p2, sal, rowptr, U1, U2, status)
+        assert int(status.item()) == st_o
+        assert np.array_equal(U1.cpu().numpy(), T1_o) and np.array_equal(U2.cpu().numpy(), T2_o)
