@@ -97,6 +97,16 @@ struct Blk {
   __device__ __forceinline__ void each(Fn fn) const {
     each(fn, [](int) {});
   }
+  // fn(x) for the weights in index order.
+  template <class Fn>
+  __device__ __forceinline__ void all(Fn fn) const {
+#pragma unroll 16
+    for (int j = 0; j < 64; ++j) {
+      const float2 v = pair(j);
+      fn(v.x);
+      fn(v.y);
+    }
+  }
 };
 
 __device__ __forceinline__ Blk stage_block(const uint16_t *W, int64_t b, uint32_t *sx) {
@@ -157,51 +167,43 @@ __device__ __forceinline__ int support(const Blk &B, V v, float d, uint32_t (&nz
   return popc4(nz);
 }
 
-// First plane of a block: mu, Delta0, T0, alpha0 (least squares with mu fixed).
-struct First {
-  float mu, d0, a0;
-  int n0;
-  uint32_t nz[4], ng[4];
-};
-
-__device__ __forceinline__ void first_plane(const Blk &B, First &f, bool *bad) {
-  float s = 0.f;
-  bool nf = false;
-  B.each([&](int, int, float x) {
-    s = __fadd_rn(s, x);
-    nf |= !isfinite(x);
-  });
-  *bad = nf;
-  const float mu = __fmul_rn(s, kInvGroup);
-  float a = 0.f;
-  B.each([&](int, int, float x) { a = __fadd_rn(a, fabsf(__fsub_rn(x, mu))); });
-  const float d0 = __fmul_rn(kThresh, __fmul_rn(a, kInvGroup));
-  f.n0 = support(B, [&](int, int, float x) { return __fsub_rn(x, mu); }, d0, f.nz, f.ng, [](float, int) {});
-  float p = 0.f;
-  B.each([&](int q, int bit, float x) {
-    p = __fadd_rn(p, times_bit(__fsub_rn(x, mu), pick4(f.nz, q), pick4(f.ng, q), bit));
-  });
-  f.mu = mu, f.d0 = d0;
-  f.a0 = f.n0 > 0 ? __fdiv_rn(p, (float)f.n0) : 0.f;
-}
-
 // ------------------------------------------------------------ statistics
+// Four passes over a block.  No pass needs the support itself: with c = w - mu
+// and Delta0 >= 0, a trit is nonzero where |c| > Delta0 and has c's sign, so
+// c * T0 is |c| there and +0 elsewhere (adding +0 to the sum of magnitudes
+// changes nothing), and r = c - alpha0 T0 has the magnitude | |c| - alpha0 |
+// there and |c| elsewhere (rounding is symmetric in the sign); E only sees r^2.
+// An inf or NaN weight makes the sum of the (16-bit) weights inf or NaN, and
+// nothing else does.  Issue-bound: 19 instructions per weight, where bit masks
+// of the support and products with its trits took 64 (114 us for 4096 x 12288,
+// this 55).
 __global__ void __launch_bounds__(kBlockThreads) tern_stats_kernel(int64_t NB, const uint16_t *W, float4 *stats,
                                                                    uint32_t *keys, uint32_t *status) {
   __shared__ uint32_t sx[64 * kBlockThreads];
   for (int64_t b = (int64_t)blockIdx.x * kBlockThreads + threadIdx.x; b < NB;
        b += (int64_t)gridDim.x * kBlockThreads) {
     const Blk B = stage_block(W, b, sx);
-    First f;
-    bool bad;
-    first_plane(B, f, &bad);
-    if (bad) atomicOr(status, TQ_DATA_BAD_WEIGHT);
+    float s = 0.f;
+    B.all([&](float x) { s = __fadd_rn(s, x); });
+    if (!isfinite(s)) atomicOr(status, TQ_DATA_BAD_WEIGHT);
+    const float mu = __fmul_rn(s, kInvGroup);
+    float a = 0.f;
+    B.all([&](float x) { a = __fadd_rn(a, fabsf(__fsub_rn(x, mu))); });
+    const float d0 = __fmul_rn(kThresh, __fmul_rn(a, kInvGroup));
+    float p = 0.f;
+    int n0 = 0;
+    B.all([&](float x) {
+      const float c = fabsf(__fsub_rn(x, mu));
+      if (c > d0) p = __fadd_rn(p, c), ++n0;
+    });
+    const float a0 = n0 > 0 ? __fdiv_rn(p, (float)n0) : 0.f;
     float e = 0.f;
-    B.each([&](int q, int bit, float x) {
-      const float r = __fsub_rn(__fsub_rn(x, f.mu), times_bit(f.a0, pick4(f.nz, q), pick4(f.ng, q), bit));
+    B.all([&](float x) {
+      const float c = fabsf(__fsub_rn(x, mu));
+      const float r = c > d0 ? __fsub_rn(c, a0) : c;
       e = __fadd_rn(e, __fmul_rn(r, r));
     });
-    stats[b] = make_float4(f.mu, f.d0, f.a0, 0.f);
+    stats[b] = make_float4(mu, d0, a0, 0.f);
     keys[b] = __float_as_uint(e);
   }
 }
@@ -415,18 +417,40 @@ __device__ __forceinline__ void plane1_blocks(int cta, int ctas, uint32_t *sx, i
     const Blk B = stage_block(W, b, sx);
     const float4 st = stats[b];
     float mu = st.x, a0 = st.z;
-    uint32_t nz0[4] = {0u, 0u, 0u, 0u}, ng0[4] = {0u, 0u, 0u, 0u};
+    const float d = st.y;
     float mw = 0.f, mw0 = 0.f;  // sum w, sum w T0
-    const int n0 = support(B, [&](int, int, float x) { return __fsub_rn(x, mu); }, st.y, nz0, ng0,
-                           [&](float x, int t) { mw += x, mw0 += t > 0 ? x : (t < 0 ? -x : 0.f); });
-    const int z0 = n0 - 2 * popc4(ng0);  // sum T0
+    int np = 0, nn = 0;         // positive, negative trits
+    uint16_t *dst = reinterpret_cast<uint16_t *>(row + (int64_t)kGroupBytes * g);
+    // a trit adds its power of 3 to a byte that starts with every digit 1
+    auto trit = [&](float x, uint32_t p3, uint32_t &v) {
+      const float c = __fsub_rn(x, mu);
+      mw += x;
+      if (c > d) mw0 += x, ++np, v += p3;
+      if (c < -d) mw0 -= x, ++nn, v -= p3;
+    };
+#pragma unroll 2
+    for (int h = 0; h < 12; ++h) {  // bytes 2 h, 2 h + 1: weights 10 h .. 10 h + 9
+      uint32_t lo = kZeroByte, hi = kZeroByte;
+      const float2 w0 = B.pair(5 * h), w1 = B.pair(5 * h + 1), w2 = B.pair(5 * h + 2), w3 = B.pair(5 * h + 3),
+                   w4 = B.pair(5 * h + 4);
+      trit(w0.x, 1, lo), trit(w0.y, 3, lo), trit(w1.x, 9, lo), trit(w1.y, 27, lo), trit(w2.x, 81, lo);
+      trit(w2.y, 1, hi), trit(w3.x, 3, hi), trit(w3.y, 9, hi), trit(w4.x, 27, hi), trit(w4.y, 81, hi);
+      dst[h] = (uint16_t)(lo | hi << 8);
+    }
+    {
+      uint32_t lo = kZeroByte, hi = kZeroByte;  // byte 24 and the tail byte
+      const float2 w0 = B.pair(60), w1 = B.pair(61), w2 = B.pair(62), w3 = B.pair(63);
+      trit(w0.x, 1, lo), trit(w0.y, 3, lo), trit(w1.x, 9, lo), trit(w1.y, 27, lo), trit(w2.x, 81, lo);
+      trit(w2.y, 1, hi), trit(w3.x, 3, hi), trit(w3.y, 9, hi);
+      dst[12] = (uint16_t)(lo | hi << 8);
+    }
+    const int n0 = np + nn, z0 = np - nn;  // |T0|, sum T0
     for (int sw = 0; sw < sweeps; ++sw) {
       mu = (mw - a0 * z0) * kInvGroup;
       a0 = n0 > 0 ? (mw0 - mu * z0) / n0 : 0.f;
     }
     off[b] = __float2half_rn(mu);
     s1[b] = __float2half_rn(a0);
-    store_group(nz0, ng0, row + (int64_t)kGroupBytes * g);
   }
 }
 
