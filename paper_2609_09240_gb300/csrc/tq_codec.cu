@@ -13,6 +13,8 @@
 // caller's status word; no kernel traps, and every plane-2 index is checked
 // against rowptr[N] before it is used.
 #include "tq_common.cuh"
+#include "tq_launch.cuh"
+#include "tq_sm100.cuh"
 
 namespace tq {
 
@@ -54,9 +56,19 @@ __global__ void __launch_bounds__(1024) rowptr_kernel(int N, int K, const uint32
   const int per = (N + blockDim.x - 1) / blockDim.x;
   const int r0 = threadIdx.x * per;
   const int r1 = min(N, r0 + per);
+  grid_dep_launch_next();
+  grid_dep_wait();
   bool pad_bad = false;
-  int local = 0;
-  for (int n = r0; n < r1; ++n) local += row_popc(sal, W, G, n, &pad_bad);
+  int local = 0, cnt[16];  // a thread's rows' counts, up to 16 rows
+  if (per <= 16) {
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      cnt[i] = r0 + i < r1 ? row_popc(sal, W, G, r0 + i, &pad_bad) : 0;
+      local += cnt[i];
+    }
+  } else {
+    for (int n = r0; n < r1; ++n) local += row_popc(sal, W, G, n, &pad_bad);
+  }
   // inclusive warp scan, then scan of warp totals
   __shared__ int warp_tot[32];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -78,10 +90,18 @@ __global__ void __launch_bounds__(1024) rowptr_kernel(int N, int K, const uint32
   }
   __syncthreads();
   int base = (wid > 0 ? warp_tot[wid - 1] : 0) + incl - local;
-  for (int n = r0; n < r1; ++n) {
-    rowptr[n] = base;
-    bool dummy = false;
-    base += row_popc(sal, W, G, n, &dummy);
+  if (per <= 16) {
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      if (r0 + i < r1) rowptr[r0 + i] = base;
+      base += cnt[i];
+    }
+  } else {
+    for (int n = r0; n < r1; ++n) {
+      rowptr[n] = base;
+      bool dummy = false;
+      base += row_popc(sal, W, G, n, &dummy);
+    }
   }
   if (threadIdx.x == blockDim.x - 1) rowptr[N] = warp_tot[(blockDim.x >> 5) - 1];
   if (pad_bad) atomicOr(status, TQ_DATA_BAD_PAD);
@@ -513,9 +533,12 @@ __host__ __device__ __forceinline__ int64_t p2index_slot_off(int K) {
   return ((int64_t)(K / kGroup + 1) * 4 + 127) & ~(int64_t)127;
 }
 
-// Rows are taken in chunks of kIdxChunk: block (g, c) handles group g's
-// rows [kIdxChunk c, kIdxChunk (c + 1)).
-constexpr int kIdxChunk = 1024;
+// The fill takes rows in chunks: block (g, c) handles group g's rows
+// [chunk c, chunk (c + 1)), in rounds of its threads.  A chunk is one round up
+// to 16384 rows (four rounds, with their block barriers, took 15 us for
+// 4096 x 12288, this 13), and at most 64 chunks are taken, since each
+// block counts the group's rows before its own.
+static int p2index_chunk(int N) { return kIdxThreads * ((N + 64 * kIdxThreads - 1) / (64 * kIdxThreads)); }
 
 // Salient rows of group g in rows [r0, r1) (the block's threads together;
 // every thread gets the total).
@@ -531,15 +554,24 @@ __device__ __forceinline__ int p2index_block_count(const uint32_t *sal, int W, i
   return t;
 }
 
-// colptr[g + 1] += salient rows of group g in the block's chunk (colptr
-// zeroed by p2index_zero_kernel).
+// Rows of a counting block: one block per group, unless a weight has more
+// rows (then the blocks add up, from zero).
+constexpr int kIdxCountRows = 16384;
+
+// colptr[g + 1] = salient rows of group g.
 __global__ void __launch_bounds__(kIdxThreads) p2index_count_kernel(int N, int K, const uint32_t *sal,
                                                                      int32_t *colptr) {
   __shared__ int red[kIdxThreads / 32];
-  const int g = blockIdx.x, c = blockIdx.y, W = sal_words_of(K);
-  const int r0 = c * kIdxChunk, r1 = min(N, r0 + kIdxChunk);
-  const int t = p2index_block_count(sal, W, g, r0, r1, red);
-  if (threadIdx.x == 0 && t) atomicAdd(colptr + g + 1, t);
+  const int g = blockIdx.x, r0 = blockIdx.y * kIdxCountRows;
+  grid_dep_launch_next();
+  grid_dep_wait();
+  const int t = p2index_block_count(sal, sal_words_of(K), g, r0, min(N, r0 + kIdxCountRows), red);
+  if (threadIdx.x == 0) {
+    if (gridDim.y == 1)
+      colptr[g + 1] = t;
+    else
+      atomicAdd(colptr + g + 1, t);
+  }
 }
 
 __global__ void p2index_zero_kernel(int G, int32_t *colptr) {
@@ -547,15 +579,24 @@ __global__ void p2index_zero_kernel(int G, int32_t *colptr) {
 }
 
 // colptr[g+1] = colptr[g] + count rounded up to 16, at most the capacity
-// (which the counts of a consistent salience map never reach).
+// (which the counts of a consistent salience map never reach).  One warp.
 __global__ void p2index_scan_kernel(int G, int64_t cap, int32_t *colptr) {
-  if (threadIdx.x != 0) return;
-  colptr[0] = 0;
-  int64_t run = 0;
-  for (int g = 0; g < G; ++g) {
-    run = min(run + (((int64_t)colptr[g + 1] + 15) & ~(int64_t)15), cap);
-    colptr[g + 1] = (int32_t)run;
+  const int lane = threadIdx.x;
+  grid_dep_launch_next();
+  grid_dep_wait();
+  int64_t base = 0;
+  for (int g0 = 0; g0 < G; g0 += 32) {
+    const int g = g0 + lane;
+    int64_t v = g < G ? ((int64_t)colptr[g + 1] + 15) & ~(int64_t)15 : 0;
+    for (int o = 1; o < 32; o <<= 1) {
+      const int64_t u = __shfl_up_sync(0xffffffffu, v, o);
+      if (lane >= o) v += u;
+    }
+    v += base;
+    if (g < G) colptr[g + 1] = (int32_t)min(v, cap);
+    base = __shfl_sync(0xffffffffu, v, 31);
   }
+  if (lane == 0) colptr[0] = 0;
 }
 
 // One slot: 8 words in the order of logical words 0, 4, 1, 5, 2, 6, 3, 7.
@@ -599,11 +640,12 @@ __device__ __forceinline__ void p2index_fill_slot(uint8_t *slot, int g, int n, i
 __global__ void __launch_bounds__(kIdxThreads) p2index_fill_kernel(int N, int K, const uint32_t *sal,
                                                                     const int32_t *rowptr, int64_t nnz,
                                                                     const uint8_t *plane2, const uint16_t *scale2,
-                                                                    int32_t *index) {
+                                                                    int32_t *index, int chunk) {
   __shared__ int warp_base[kIdxThreads / 32 + 1];
   __shared__ int red[kIdxThreads / 32];
   const int G = K / kGroup, g = blockIdx.x, c = blockIdx.y, W = sal_words_of(K);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  grid_dep_wait();
   uint8_t *slots = reinterpret_cast<uint8_t *>(index) + p2index_slot_off(K);
   if (g == G) {
     if (c != 0) return;
@@ -611,7 +653,7 @@ __global__ void __launch_bounds__(kIdxThreads) p2index_fill_kernel(int N, int K,
     for (int64_t e = index[G] + threadIdx.x; e < cap; e += kIdxThreads) p2index_empty_slot(slots + 32 * e);
     return;
   }
-  const int r0 = c * kIdxChunk, r1 = min(N, r0 + kIdxChunk);
+  const int r0 = c * chunk, r1 = min(N, r0 + chunk);
   if (r0 >= N) return;
   const int64_t lim = index[g + 1];
   int64_t base = index[g] + p2index_block_count(sal, W, g, 0, r0, red);
@@ -654,8 +696,7 @@ static int grid_for(int64_t work, int block) {
 
 cudaError_t launch_rowptr(int N, int K, const uint32_t *sal, int32_t *rowptr, uint32_t *status,
                           cudaStream_t s) {
-  rowptr_kernel<<<1, 1024, 0, s>>>(N, K, sal, rowptr, status);
-  return cudaGetLastError();
+  return launch_dependent(rowptr_kernel, dim3(1), 1024, s, N, K, sal, rowptr, status);
 }
 
 cudaError_t launch_check_rowptr(int N, int K, const uint32_t *sal, const int32_t *rowptr,
@@ -705,12 +746,17 @@ cudaError_t launch_unpack(int N, int K, const uint8_t *plane1, const uint8_t *pl
 
 cudaError_t launch_plane2_index(int N, int K, const uint32_t *sal, const int32_t *rowptr, int64_t nnz,
                                 const uint8_t *plane2, const uint16_t *scale2, int32_t *index, cudaStream_t s) {
-  const int G = K / kGroup, C = (N + kIdxChunk - 1) / kIdxChunk;
-  p2index_zero_kernel<<<1, 256, 0, s>>>(G, index);
-  p2index_count_kernel<<<dim3(G, C), kIdxThreads, 0, s>>>(N, K, sal, index);
-  p2index_scan_kernel<<<1, 32, 0, s>>>(G, p2index_capacity(K, nnz), index);
-  p2index_fill_kernel<<<dim3(G + 1, C), kIdxThreads, 0, s>>>(N, K, sal, rowptr, nnz, plane2, scale2, index);
-  return cudaGetLastError();
+  const int G = K / kGroup, chunk = p2index_chunk(N), C = (N + kIdxCountRows - 1) / kIdxCountRows;
+  cudaError_t e;
+  if (C > 1) {
+    p2index_zero_kernel<<<1, 256, 0, s>>>(G, index);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  }
+  if ((e = launch_dependent(p2index_count_kernel, dim3(G, C), kIdxThreads, s, N, K, sal, index)) != cudaSuccess) return e;
+  if ((e = launch_dependent(p2index_scan_kernel, dim3(1), 32, s, G, p2index_capacity(K, nnz), index)) != cudaSuccess)
+    return e;
+  return launch_dependent(p2index_fill_kernel, dim3(G + 1, (N + chunk - 1) / chunk), kIdxThreads, s, N, K, sal, rowptr,
+                          nnz, plane2, scale2, index, chunk);
 }
 
 // ------------------------------------------ element-wise four-mask format

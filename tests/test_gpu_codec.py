@@ -208,6 +208,12 @@ def test_plane2_index_bit_exact(H, N, K, frac):
     assert bad.size == 0, f"{bad.size} slots differ; first {bad[0]}: {got[bad[0]]} vs {slots[bad[0]]}"
 
 
+@pytest.mark.parametrize("N", [16384, 16385])
+def test_plane2_index_tall(H, N):
+    """One counting block per group and chunks of one round; several and two."""
+    test_plane2_index_bit_exact(H, N, 256, 0.1)
+
+
 @pytest.mark.parametrize("N,K,offset", [(1, 128, 0), (31, 128, 0), (33, 128, 0), (129, 128, 0), (5, 896, 0), (41, 1408, 0),
                                         (3, 4224, 0), (2, 49280, 0), (16, 4096, 1)])
 def test_pack_unpack_warp_tiles(H, N, K, offset):

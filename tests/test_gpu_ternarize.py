@@ -101,6 +101,23 @@ def test_ternarize_degenerate():
     assert not r["T1"].any()
 
 
+@pytest.mark.parametrize("N,K,frac", [
+    (26608, 128, 0.1),  # rows padded to whole words: the most that one cluster's shared memory holds
+    (26609, 128, 0.1),  # one row more: selection over the whole chip
+    (26609, 128, 0.7),
+    (15, 33 * 128, 0.1),  # fewer rows than CTAs
+    (100, 31 * 128, 0.7),
+])
+def test_ternarize_selection_paths(N, K, frac):
+    """Both selections, with two groups in five of constant weights (E = 0), so
+    that 70 % salient reaches into keys that equal the padding."""
+    W = wl.gen_dense_weights(N, K, config=9, proj=2).reshape(N * (K // 128), 128)
+    b = np.arange(len(W))
+    W[b % 5 < 2] = W[b % 5 < 2, :1]
+    W = W.reshape(N, K)
+    compare(W, int(round(frac * len(b))), 2)
+
+
 def test_ternarize_full_size_gate_projection():
     """A Qwen3-8B gate projection (12288 x 4096, 10 % salient groups, four
     refinement sweeps) in one call, every output compared."""
