@@ -569,18 +569,34 @@ __global__ void __launch_bounds__((WD + 1) * 32, 1)
 }
 
 // ------------------------------------------------------------ sequence
+// floor(v c / n) without a 64-bit product or quotient (c < n <= 256).
+__device__ __forceinline__ int share_at(int v, int c, int n) {
+  const int q = (int)((unsigned)v / (unsigned)n);
+  return q * c + (int)((unsigned)(v - q * n) * (unsigned)c / (unsigned)n);
+}
+
 // Dependency-ordered sequence of problems (one token): problem p + 1 starts
 // only after every CTA has finished problem p, as the layers of a model need
 // (q/k/v, then o, then gate/up, then down, layer after layer; the attention,
 // norms and activation between them are outside this library).  One
 // persistent launch: for each problem every CTA takes its share of the
-// second-plane tiles and then of the 256-row tiles' stage units (tiles cut so
-// that the problem's units cover the CTAs), adding everything into y2 (fp32
-// atomics, zeroed by the prep kernel); a grid-wide barrier (a counter in the
-// workspace, bounded by the wall-time limit) ends the problem, after which
-// every CTA converts its slice of y2 into y.  The producer warp streams the
-// stages without waiting at the barriers (weights do not depend on earlier
-// problems).  barrier_extra > 0 makes every barrier wait for CTAs that do not
+// 256-row tiles' stage units (tiles cut so that the problem's units cover the
+// CTAs; the decode warps) and of the second-plane tiles (kSeqP2 warps of their
+// own, beside them), adding everything into y2 (fp32 atomics, zeroed by the
+// prep kernel); a grid-wide barrier (a counter in the workspace, bounded by
+// the wall-time limit) ends the problem, after which every CTA converts its
+// slice of y2 into y.
+//
+// A problem is one or two stages per SM, so its time is a chain of latencies,
+// and everything that does not depend on earlier problems is kept out of it:
+// the producer warp streams the stages without waiting at the barriers, the
+// second-plane warps have their first tiles' group, operands and records in
+// registers when the barrier opens, the decode warps the next problem's
+// parameters and walk (worked out from a cold parameter space after the
+// barrier they took 3500 cycles a problem), and a row of y is loaded after the
+// barrier and stored after the next problem's stages.  One Qwen3-8B step of
+// 144 problems: 1.14 ms; with the second plane done by the decode warps before
+// their stages, and all of this after the barrier, 1.61.  barrier_extra > 0 makes every barrier wait for CTAs that do not
 // exist, so that its bounded wait runs out (the failure-path self-test).
 struct SeqWalk {
   const BatchParams *bp;
@@ -588,13 +604,13 @@ struct SeqWalk {
   __device__ void enter() {
     const Problem &P = bp->prob[p];
     const int G = P.K / kGroup, tiles = (P.N + kRows - 1) / kRows;
-    const int64_t share = ((int64_t)tiles * G + ctas - 1) / ctas;
-    const int split = share >= G ? 0 : (int)(share < 1 ? 1 : share);
+    // the CTA's fair share of the tiles' groups (whole tiles from one tile up)
+    const int share = tiles >= ctas ? G : (tiles * G + ctas - 1) / ctas;
+    const int split = share >= G ? 0 : share < 1 ? 1 : share;
     u = unit_parts(P.K, 8, split);
     nst = nstages(P.K, 8);
-    const int64_t U = (int64_t)tiles * u;
-    unit = (int)(U * cta / ctas);
-    u_end = (int)(U * (cta + 1) / ctas);
+    unit = share_at(tiles * u, cta, ctas);
+    u_end = share_at(tiles * u, cta + 1, ctas);
     if (unit < u_end) locate();
   }
   __device__ void locate() {
@@ -625,45 +641,65 @@ __device__ __forceinline__ int ld_acquire(const int32_t *p) {
   return v;
 }
 
-// A decode warp's share of problem P's second-plane tiles (one token): the
-// CTA's contiguous share of the index's 16-entry tiles, cut among the WD
-// decode warps; runs of tiles of one group go through mm::p2_tiles with the
-// group's activation fragment of the per-group layout.
-template <int WD>
-__device__ __forceinline__ void second_plane_share(const Problem &P, int cta, int ctas, int warp, int lane,
-                                                   uint32_t tag) {
-  const int G = P.K / kGroup, c = lane & 3;
-  const int T2 = __ldg(P.p2idx + G) >> 4;  // tiles (group starts are multiples of 16 entries)
-  const int lo = (int)((int64_t)T2 * cta / ctas), hi = (int)((int64_t)T2 * (cta + 1) / ctas);
-  const int wlo = lo + (hi - lo) * warp / WD, whi = lo + (hi - lo) * (warp + 1) / WD;
-  for (int t = wlo; t < whi;) {
+constexpr int kSeqP2 = 3;  // second-plane warps
+
+// A second-plane warp's share of problem P's tiles (one token): the CTA's
+// contiguous share of the index's 16-entry tiles, cut among the kSeqP2 warps,
+// in runs of tiles of one group (mm::p2_tiles with the group's activation
+// fragment of the per-group layout).  start() fetches what the first run
+// needs before the barrier that lets it begin: all of it is weights and
+// operands of the prep kernel.
+struct SeqP2 {
+  int t, end, n, g;
+  const unsigned char *src;
+  uint32_t b[20];
+  float2 Cv;
+  uint2 pre[mm::kCDepth][2];
+  __device__ __forceinline__ void load_run(const Problem &P, int lane) {
+    n = 0;
+    if (t >= end) return;
     // the tile's group: the last g with colptr[g] <= 16 t
-    int g = 0;
-    for (int step = 1 << (31 - __clz(G)); step >= 1; step >>= 1)
-      if (g + step < G && __ldg(P.p2idx + g + step) <= 16 * t) g += step;
-    const int64_t e0 = __ldg(P.p2idx + g);
-    const int n = min(whi, __ldg(P.p2idx + g + 1) >> 4) - t;
-    if (n <= 0) break;  // malformed index: stop rather than loop
+    const int G = P.K / kGroup, c = lane & 3;
+    g = 0;
+#pragma unroll 4
+    for (int i = 1 + lane; i - lane < G; i += 32)
+      g += __popc(__ballot_sync(0xffffffffu, i < G && __ldg(P.p2idx + min(i, G)) <= 16 * t));
+    n = min(end, __ldg(P.p2idx + g + 1) >> 4) - t;
+    if (n <= 0) return;  // malformed index: the share ends here
+    src = mm::p2_src(P, g % mm::kStageG, 16 * (int64_t)t, 0, lane);
+    mm::p2_first(src, n, pre);
     const unsigned char *Bg = P.wsB + (int64_t)g * mm::kBTok + c * mm::kBLane;
-    uint32_t b[20];
 #pragma unroll
     for (int cp = 0; cp < mm::kCP; ++cp) {
       const uint4 v = __ldg(reinterpret_cast<const uint4 *>(Bg + cp * 4 * mm::kBLane));
       b[4 * cp] = v.x, b[4 * cp + 1] = v.y, b[4 * cp + 2] = v.z, b[4 * cp + 3] = v.w;
     }
-    const float2 Cv = __ldg(reinterpret_cast<const float2 *>(P.wsCS + (int64_t)g * (mm::kCSGroup / 4)));
-    mm::p2_tiles<true, false>(P, 1, g % mm::kStageG, e0, t - (int)(e0 >> 4), n, b, b, Cv, Cv, lane, tag);
-    t += n;
+    Cv = __ldg(reinterpret_cast<const float2 *>(P.wsCS + (int64_t)g * (mm::kCSGroup / 4)));
   }
-}
+  __device__ __forceinline__ void start(const Problem &P, int cta, int ctas, int pw, int lane) {
+    t = end = n = 0;
+    if (P.nnz <= 0) return;
+    const int T2 = __ldg(P.p2idx + P.K / kGroup) >> 4;  // tiles (group starts are multiples of 16 entries)
+    const int lo = share_at(T2, cta, ctas), hi = share_at(T2, cta + 1, ctas);
+    t = lo + (hi - lo) * pw / kSeqP2, end = lo + (hi - lo) * (pw + 1) / kSeqP2;
+    load_run(P, lane);
+  }
+  __device__ __forceinline__ void run(const Problem &P, int lane, uint32_t tag) {
+    while (n > 0) {
+      mm::p2_tiles<true, false>(P, 1, g % mm::kStageG, src, n, pre, b, b, Cv, Cv, lane, tag);
+      t += n;
+      load_run(P, lane);
+    }
+  }
+};
 
 // The CTA's share of problem P's second-plane records (the tiles that
-// second_plane_share gives it) into L2, one bulk prefetch: they are weights,
+// SeqP2 gives it) into L2, one bulk prefetch: they are weights,
 // so they can be fetched while the problem before P still runs.
 __device__ __forceinline__ void prefetch_second_plane(const Problem &P, int cta, int ctas) {
   const int G = P.K / kGroup;
   const int T2 = __ldg(P.p2idx + G) >> 4;
-  const int lo = (int)((int64_t)T2 * cta / ctas), hi = (int)((int64_t)T2 * (cta + 1) / ctas);
+  const int lo = share_at(T2, cta, ctas), hi = share_at(T2, cta + 1, ctas);
   if (hi <= lo) return;
   const unsigned char *slots = reinterpret_cast<const unsigned char *>(P.p2idx) + mm::c_slot_off(P.K);
   asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(slots + (int64_t)lo * 512),
@@ -672,7 +708,7 @@ __device__ __forceinline__ void prefetch_second_plane(const Problem &P, int cta,
 }
 
 template <bool F32>
-__global__ void __launch_bounds__((kWD1 + 1) * 32, 1)
+__global__ void __launch_bounds__((kWD1 + 1 + kSeqP2) * 32, 1)
     gemv_seq_kernel(const __grid_constant__ BatchParams bp, int32_t barrier_extra) {
   constexpr int SG = 8, MB = 1, WD = kWD1, TL = kTL1;
   using C = Cfg<SG>;
@@ -685,7 +721,10 @@ __global__ void __launch_bounds__((kWD1 + 1) * 32, 1)
   }
   Bars *bars = reinterpret_cast<Bars *>(dyn + C::kOffBars);
   volatile int32_t *abort_ = &bars->abort_;
-  setup_cta<SG, WD>(dyn, tid, (WD + 1) * 32);
+  // named barriers of the decode and second-plane warps: a problem's work in
+  // this CTA is done (1), in every CTA (2)
+  constexpr int kWorkers = (WD + kSeqP2) * 32;
+  setup_cta<SG, WD>(dyn, tid, (WD + 1 + kSeqP2) * 32);
   __syncthreads();
   grid_dep_wait();  // the prep kernel's operands, maps, zeroed y2 and counter
   int32_t *counter = reinterpret_cast<int32_t *>(static_cast<unsigned char *>(bp.prob[0].map()) + 448);
@@ -702,11 +741,19 @@ __global__ void __launch_bounds__((kWD1 + 1) * 32, 1)
     uint32_t bz[kBSets][4] = {};
     uint32_t buf = 0, phase = 0;
     SeqWalk w(&bp, blockIdx.x, gridDim.x);
-    for (bool more = true; more; more = w.next_problem()) {
+    // rows [r0, r1) of a finished problem whose y this CTA stores; the
+    // thread's first row waits in yv
+    void *yp = nullptr;
+    int r0 = 0, r1 = 0;
+    float yv = 0.f;
+    auto y_store = [&](int n, float v) {
+      if (F32)
+        static_cast<float *>(yp)[n] = v;
+      else
+        static_cast<__half *>(yp)[n] = __float2half_rn(v);
+    };
+    for (bool more = true; more;) {
       const Problem &P = w.P();
-      if (warp == 0 && lane == 0 && w.p + 1 < bp.count && bp.prob[w.p + 1].nnz > 0)
-        prefetch_second_plane(bp.prob[w.p + 1], blockIdx.x, gridDim.x);
-      if (P.nnz > 0) second_plane_share<WD>(P, blockIdx.x, gridDim.x, warp, lane, tag);
       bool ok = true;
       for (; w.has_stage(); w.next_stage()) {
         ok = __all_sync(0xffffffffu, mm::wait_or_abort(&bars->full[buf], phase, abort_));
@@ -727,12 +774,25 @@ __global__ void __launch_bounds__((kWD1 + 1) * 32, 1)
         }
         if (++buf == (uint32_t)kNS) buf = 0, phase ^= 1u;
       }
+      if (r0 + tid < r1) y_store(r0 + tid, yv);  // of the problem before
       // the problem's barrier: every CTA's additions into y2 are done
-      named_bar(1, WD * 32);
+      if (warp != 0) {
+        named_bar_arrive(1, kWorkers);
+      } else {
+        named_bar(1, kWorkers);
+        if (lane == 0 && ok && !*abort_) {
+          __threadfence();
+          atomicAdd(counter, 1);
+        }
+        __syncwarp();
+      }
+      // what the next problem needs of the parameters, while the others finish
+      const int target = (w.p + 1) * ((int)gridDim.x + barrier_extra);
+      const float *y2 = P.y2();
+      yp = P.y;
+      r0 = share_at(P.N, blockIdx.x, gridDim.x), r1 = share_at(P.N, blockIdx.x + 1, gridDim.x);
+      more = w.next_problem();
       if (warp == 0 && lane == 0 && ok && !*abort_) {
-        __threadfence();
-        atomicAdd(counter, 1);
-        const int target = (w.p + 1) * ((int)gridDim.x + barrier_extra);
         const uint64_t t0 = global_ns();
         while (ld_acquire(counter) < target) {
           if (*abort_) break;
@@ -741,23 +801,22 @@ __global__ void __launch_bounds__((kWD1 + 1) * 32, 1)
             *abort_ = 1;
             break;
           }
-          __nanosleep(32);  // 1.603 ms per Qwen3-8B step against 1.610 with 128 ns (spinning: 1.611)
+          __nanosleep(32);  // (measured faster than 128 ns and than spinning)
         }
-        __threadfence();
       }
+      __syncwarp();
       // stop together: the flag may be raised (by the producer) while
       // the warps read it, so they decide by one reduction over the barrier
-      if (named_bar_any(1, WD * 32, *abort_ != 0)) break;
-      // this CTA's slice of the problem's output
-      const int r0 = (int)((int64_t)P.N * blockIdx.x / gridDim.x), r1 = (int)((int64_t)P.N * (blockIdx.x + 1) / gridDim.x);
-      for (int n = r0 + warp * 32 + lane; n < r1; n += WD * 32) {
-        const float v = __ldcg(P.y2() + n);
-        if (F32)
-          static_cast<float *>(P.y)[n] = v;
-        else
-          static_cast<__half *>(P.y)[n] = __float2half_rn(v);
+      if (named_bar_any(2, kWorkers, *abort_ != 0)) {
+        r1 = 0;
+        break;
       }
+      // this CTA's slice of the problem's output: the thread's first row is
+      // loaded here and stored after the next problem's stages
+      if (r0 + tid < r1) yv = __ldcg(y2 + r0 + tid);
+      for (int n = r0 + tid + WD * 32; n < r1; n += WD * 32) y_store(n, __ldcg(y2 + n));
     }
+    if (r0 + tid < r1) y_store(r0 + tid, yv);
   } else if (warp == WD) {
     // ========================================================== producer
     uint32_t buf = 0, phase = 0, q = 0;
@@ -780,6 +839,21 @@ __global__ void __launch_bounds__((kWD1 + 1) * 32, 1)
     if (lane == 0) {
       for (uint32_t k = (q > (uint32_t)kNS ? q - kNS : 0); k < q; ++k) mbar_wait(&bars->full[k % kNS], (k / kNS) & 1u);
     }
+  } else {
+    // ====================================================== second plane
+    SeqP2 sp;
+    const uint32_t tag = kLutShared | ((uint32_t)lane << 2);
+    bool stop = false;
+    for (int p = 0; p < bp.count && !stop; ++p) {
+      const Problem &P = bp.prob[p];
+      sp.start(P, blockIdx.x, gridDim.x, warp - WD - 1, lane);
+      if (p > 0 && (stop = named_bar_any(2, kWorkers, *abort_ != 0))) break;
+      if (warp == WD + 1 && lane == 0 && p + 1 < bp.count && bp.prob[p + 1].nnz > 0)
+        prefetch_second_plane(bp.prob[p + 1], blockIdx.x, gridDim.x);
+      sp.run(P, lane, tag);
+      named_bar_arrive(1, kWorkers);
+    }
+    if (!stop) named_bar_any(2, kWorkers, *abort_ != 0);
   }
   __syncthreads();
 }
@@ -1090,7 +1164,7 @@ cudaError_t launch_gemv_seq(const BatchParams &bp, int num_sms, int barrier_extr
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(ctas);
-  cfg.blockDim = dim3((g4::kWD1 + 1) * 32);
+  cfg.blockDim = dim3((g4::kWD1 + 1 + g4::kSeqP2) * 32);
   cfg.dynamicSmemBytes = g4::kDynBytes;
   cfg.stream = s;
   cudaLaunchAttribute attr[1];

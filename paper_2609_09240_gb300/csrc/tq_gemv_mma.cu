@@ -1018,7 +1018,10 @@ __global__ void __launch_bounds__(c_threads(TWO), 1)
       }
       Cv2 = __ldg(reinterpret_cast<const float2 *>(csg + 16 + 2 * c));
     }
-    p2_tiles<ONE, TWO>(P, MB, GL, e0, t0, n, b, b2, Cv, Cv2, lane, tag);
+    const unsigned char *src = p2_src(P, GL, e0, t0, lane);
+    uint2 pre[kCDepth][2];
+    p2_first(src, n, pre);
+    p2_tiles<ONE, TWO>(P, MB, GL, src, n, pre, b, b2, Cv, Cv2, lane, tag);
   }
 }
 

@@ -87,35 +87,44 @@ __device__ __forceinline__ int64_t c_slot_off(int K) { return ((int64_t)(K / kGr
 
 constexpr int kCDepth = 2;  // tiles in flight per warp (in registers)
 
-// n consecutive 16-entry tiles of group g's entries (from entry e0 + 16 t0),
-// as m16 tiles of one warp: lane (r, c) loads slot words 2 jw, 2 jw + 1 of
-// entries r and r + 8 (its two window words, one 8-byte load per entry; a
-// quad's loads cover the slot), decodes them with the lane-replicated table
-// (tag = table base | lane * 4) and, after the MMAs with the group's B words
-// b (b2: tokens 8..15) and corrections Cv (Cv2), takes the entries' rows
-// and s2 from the quad's lanes that hold them and adds s2 (D - C) to y2.
+// The slot words of the lane in the first tile of a run (p2_tiles) of tiles
+// of a group at stage position GL; the run's tile t is 512 t bytes further.
+__device__ __forceinline__ const unsigned char *p2_src(const Problem &P, int GL, int64_t e0, int t0, int lane) {
+  const int jw = ((lane & 3) - win_start(GL)) & 3;
+  return reinterpret_cast<const unsigned char *>(P.p2idx) + c_slot_off(P.K) +
+         (e0 + 16 * (int64_t)t0 + (lane >> 2)) * 32 + jw * 8;
+}
+// The slot words of a run's first kCDepth tiles.
+__device__ __forceinline__ void p2_first(const unsigned char *src, int n, uint2 (&pre)[kCDepth][2]) {
+#pragma unroll
+  for (int k = 0; k < kCDepth; ++k) {
+    pre[k][0] = pre[k][1] = make_uint2(0u, 0u);
+    if (k < n) {
+      pre[k][0] = __ldg(reinterpret_cast<const uint2 *>(src + k * 512));
+      pre[k][1] = __ldg(reinterpret_cast<const uint2 *>(src + k * 512 + 256));
+    }
+  }
+}
+
+// n consecutive 16-entry tiles of group g's entries (src: p2_src, pre: the
+// first tiles' words), as m16 tiles of one warp: lane (r, c) loads slot words
+// 2 jw, 2 jw + 1 of entries r and r + 8 (its two window words, one 8-byte load
+// per entry; a quad's loads cover the slot), decodes them with the
+// lane-replicated table (tag = table base | lane * 4) and, after the MMAs with
+// the group's B words b (b2: tokens 8..15) and corrections Cv (Cv2), takes the
+// entries' rows and s2 from the quad's lanes that hold them and adds
+// s2 (D - C) to y2.
 template <bool ONE, bool TWO>
-__device__ __forceinline__ void p2_tiles(const Problem &P, int MB, int GL, int64_t e0, int t0, int n,
-                                         const uint32_t *b, const uint32_t *b2, float2 Cv, float2 Cv2, int lane,
-                                         uint32_t tag) {
-  const int g16 = lane >> 2, c = lane & 3, quad = lane & ~3;
+__device__ __forceinline__ void p2_tiles(const Problem &P, int MB, int GL, const unsigned char *src, int n,
+                                         uint2 (&pre)[kCDepth][2], const uint32_t *b, const uint32_t *b2, float2 Cv,
+                                         float2 Cv2, int lane, uint32_t tag) {
+  const int c = lane & 3, quad = lane & ~3;
     // lane c's window words jw and jw + 4 are slot words 2 jw, 2 jw + 1; the row is the second
     // word of the lane with jw = 3, s2 a half of the first word of jw = 0 (record at byte 2)
     // or of the second word of jw = 2 (record at byte 0)
-    const int ws = win_start(GL), jw = (c - ws) & 3, odd = GL & 1;
+    const int ws = win_start(GL), odd = GL & 1;
     const int c_row = quad + ((3 + ws) & 3), c_s2 = quad + (((odd ? 0 : 2) + ws) & 3);
-    const unsigned char *src = reinterpret_cast<const unsigned char *>(P.p2idx) + c_slot_off(P.K) +
-                               (e0 + 16 * (int64_t)t0 + g16) * 32 + jw * 8;
     float *y2 = P.y2();
-    uint2 pre[kCDepth][2];
-#pragma unroll
-    for (int k = 0; k < kCDepth; ++k) {
-      pre[k][0] = pre[k][1] = make_uint2(0u, 0u);
-      if (k < n) {
-        pre[k][0] = __ldg(reinterpret_cast<const uint2 *>(src + k * 512));
-        pre[k][1] = __ldg(reinterpret_cast<const uint2 *>(src + k * 512 + 256));
-      }
-    }
     for (int t = 0; t < n; t += kCDepth) {
 #pragma unroll
       for (int k = 0; k < kCDepth; ++k) {

@@ -50,6 +50,12 @@ def test_sequence_mixed_shapes(H):
     _run(H, shapes, 0.1, config=8)
 
 
+def test_sequence_tall(H):
+    """More rows per CTA than decode threads, and second-plane shares that run
+    over many groups."""
+    _run(H, [(80_001, 128), (520, 5120), (80_001, 128)], 0.5, config=8, rows_per=500)
+
+
 def test_sequence_no_second_plane(H):
     _run(H, [(512, 1024), (256, 2048), (1000, 1152)], 0.0, config=8)
 
