@@ -651,6 +651,11 @@ constexpr int kSeqP2 = 3;  // second-plane warps
 // operands of the prep kernel.
 struct SeqP2 {
   int t, end, n, g;
+  // the index's tiles (group starts are multiples of 16 entries), clamped into it
+  static __device__ __forceinline__ int tiles_of(const Problem &P) {
+    const int e = __ldg(P.p2idx + P.K / kGroup);
+    return (int)(min((int64_t)max(e, 0), mm::c_capacity(P.K, P.nnz)) >> 4);
+  }
   const unsigned char *src;
   uint32_t b[20];
   float2 Cv;
@@ -679,7 +684,7 @@ struct SeqP2 {
   __device__ __forceinline__ void start(const Problem &P, int cta, int ctas, int pw, int lane) {
     t = end = n = 0;
     if (P.nnz <= 0) return;
-    const int T2 = __ldg(P.p2idx + P.K / kGroup) >> 4;  // tiles (group starts are multiples of 16 entries)
+    const int T2 = tiles_of(P);
     const int lo = share_at(T2, cta, ctas), hi = share_at(T2, cta + 1, ctas);
     t = lo + (hi - lo) * pw / kSeqP2, end = lo + (hi - lo) * (pw + 1) / kSeqP2;
     load_run(P, lane);
@@ -697,8 +702,7 @@ struct SeqP2 {
 // SeqP2 gives it) into L2, one bulk prefetch: they are weights,
 // so they can be fetched while the problem before P still runs.
 __device__ __forceinline__ void prefetch_second_plane(const Problem &P, int cta, int ctas) {
-  const int G = P.K / kGroup;
-  const int T2 = __ldg(P.p2idx + G) >> 4;
+  const int T2 = SeqP2::tiles_of(P);
   const int lo = share_at(T2, cta, ctas), hi = share_at(T2, cta + 1, ctas);
   if (hi <= lo) return;
   const unsigned char *slots = reinterpret_cast<const unsigned char *>(P.p2idx) + mm::c_slot_off(P.K);
@@ -707,7 +711,10 @@ __device__ __forceinline__ void prefetch_second_plane(const Problem &P, int cta,
                : "memory");
 }
 
-template <bool F32>
+// ONE: a single problem, as a call of its own.  Such a call may share the GPU
+// with others, so its CTAs wait for none of each other: the last one to finish
+// (a ticket from the counter) stores all of y.
+template <bool F32, bool ONE>
 __global__ void __launch_bounds__((kWD1 + 1 + kSeqP2) * 32, 1)
     gemv_seq_kernel(const __grid_constant__ BatchParams bp, int32_t barrier_extra) {
   constexpr int SG = 8, MB = 1, WD = kWD1, TL = kTL1;
@@ -774,6 +781,7 @@ __global__ void __launch_bounds__((kWD1 + 1 + kSeqP2) * 32, 1)
         }
         if (++buf == (uint32_t)kNS) buf = 0, phase ^= 1u;
       }
+      if constexpr (ONE) break;
       if (r0 + tid < r1) y_store(r0 + tid, yv);  // of the problem before
       // the problem's barrier: every CTA's additions into y2 are done
       if (warp != 0) {
@@ -816,7 +824,36 @@ __global__ void __launch_bounds__((kWD1 + 1 + kSeqP2) * 32, 1)
       if (r0 + tid < r1) yv = __ldcg(y2 + r0 + tid);
       for (int n = r0 + tid + WD * 32; n < r1; n += WD * 32) y_store(n, __ldcg(y2 + n));
     }
-    if (r0 + tid < r1) y_store(r0 + tid, yv);
+    if constexpr (ONE) {
+      named_bar(1, kWorkers);
+      bool last = false;
+      if (tid == 0 && !*abort_) {
+        __threadfence();
+        last = atomicAdd(counter, 1) == (int)gridDim.x - 1;
+        __threadfence();
+      }
+      if (named_bar_any(2, WD * 32, last)) {
+        const Problem &P = bp.prob[0];
+        const float *y2 = P.y2();
+        yp = P.y;
+        constexpr int B = 16;  // rows a thread has in flight
+        for (int n0 = tid; n0 < P.N; n0 += B * WD * 32) {
+          float v[B];
+#pragma unroll
+          for (int i = 0; i < B; ++i) {
+            const int n = n0 + i * WD * 32;
+            v[i] = n < P.N ? __ldcg(y2 + n) : 0.f;
+          }
+#pragma unroll
+          for (int i = 0; i < B; ++i) {
+            const int n = n0 + i * WD * 32;
+            if (n < P.N) y_store(n, v[i]);
+          }
+        }
+      }
+    } else if (r0 + tid < r1) {
+      y_store(r0 + tid, yv);
+    }
   } else if (warp == WD) {
     // ========================================================== producer
     uint32_t buf = 0, phase = 0, q = 0;
@@ -853,7 +890,7 @@ __global__ void __launch_bounds__((kWD1 + 1 + kSeqP2) * 32, 1)
       sp.run(P, lane, tag);
       named_bar_arrive(1, kWorkers);
     }
-    if (!stop) named_bar_any(2, kWorkers, *abort_ != 0);
+    if (!ONE && !stop) named_bar_any(2, kWorkers, *abort_ != 0);
   }
   __syncthreads();
 }
@@ -1156,10 +1193,12 @@ cudaError_t launch_gemv_p2r(const BatchParams &bp, int num_sms, int32_t *counter
 
 // The dependency-ordered sequence kernel (one token), launched
 // programmatically after its prep kernel.
-cudaError_t launch_gemv_seq(const BatchParams &bp, int num_sms, int barrier_extra, cudaStream_t s) {
-  if (bp.M != 1 || bp.count < 1) return cudaErrorInvalidValue;
+// (one: the variant whose CTAs do not wait for one another, one problem.)
+cudaError_t launch_gemv_seq(const BatchParams &bp, int num_sms, int barrier_extra, bool one, cudaStream_t s) {
+  if (bp.M != 1 || bp.count < 1 || (one && bp.count != 1)) return cudaErrorInvalidValue;
   const int ctas = std::min(num_sms, 256);
-  auto kern = bp.out_f32 ? g4::gemv_seq_kernel<true> : g4::gemv_seq_kernel<false>;
+  auto kern = one ? (bp.out_f32 ? g4::gemv_seq_kernel<true, true> : g4::gemv_seq_kernel<false, true>)
+                  : (bp.out_f32 ? g4::gemv_seq_kernel<true, false> : g4::gemv_seq_kernel<false, false>);
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, g4::kDynBytes);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};

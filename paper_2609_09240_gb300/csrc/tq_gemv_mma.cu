@@ -1338,7 +1338,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 cudaError_t launch_gemv_g4(const BatchParams &bp, int num_sms, cudaStream_t s);
 cudaError_t launch_gemv_p2r(const BatchParams &bp, int num_sms, int32_t *counter, cudaStream_t s);
 int g4_split_for(const BatchParams &bp, int num_sms);
-cudaError_t launch_gemv_seq(const BatchParams &bp, int num_sms, int barrier_extra, cudaStream_t s);
+cudaError_t launch_gemv_seq(const BatchParams &bp, int num_sms, int barrier_extra, bool one, cudaStream_t s);
 
 static int num_sms_mm() {
   static int n = 0;
@@ -1520,8 +1520,27 @@ static cudaError_t launch_mm(const BatchParams &bp, cudaStream_t s) {
   return cudaSuccess;
 }
 
+static cudaError_t launch_sequence(const BatchParams &bp_in, int barrier_extra, bool one, cudaStream_t s);
+
+// One token, one weight with an indexed second plane: both planes in one
+// kernel (the dependency-ordered one's variant for a single problem), instead
+// of one after the other in two.  10 % salient, as calls in a row: 2560 x 4096
+// 13.2 us against 17.6, 12288 x 4096 16.9 against 23.7, 49152 x 4096 33.8
+// against 42.5; 151936 x 4096 84 against 97, but 167 against 163 with 30 %
+// salient (its three second-plane warps then bind), so larger weights keep the
+// two kernels.  Without a second plane the first plane's kernel alone is as
+// fast (1024 x 2560: 11.1 against 12.3).
+static bool one_launch(const BatchParams &bp) {
+  if (!g4::takes(bp) || bp.M != 1 || bp.count != 1) return false;
+  const Problem &P = bp.prob[0];
+  if (P.nnz <= 0 || !P.p2idx) return false;
+  const int64_t units = (int64_t)((P.N + g4::kRows - 1) / g4::kRows) * g4::nstages(P.K, 8);
+  return units <= 16 * (int64_t)num_sms_mm();
+}
+
 template <bool F32>
 static cudaError_t launch_mm_one(const BatchParams &bp_in, cudaStream_t s) {
+  if (one_launch(bp_in)) return launch_sequence(bp_in, 0, true, s);
   // the batch with the M <= 2 kernel's tile split filled in
   thread_local BatchParams bp;
   bp = bp_in;
@@ -1630,12 +1649,13 @@ static cudaError_t launch_mm_one(const BatchParams &bp_in, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-// The dependency-ordered sequence (one token): prep (operands of every
+// The dependency-ordered sequence (one token; one: a single problem, without
+// the grid's barriers): prep (operands of every
 // problem, maps, zeroed y2 and barrier counter), then the persistent
 // sequence kernel (tq_gemv_g4.cu).  Every problem with a second plane must
 // carry its index.  A sequence's problems must fit one set of tensor-map
 // templates (cudaErrorNotSupported otherwise).
-cudaError_t launch_gemv_sequence(const BatchParams &bp_in, int barrier_extra, cudaStream_t s) {
+static cudaError_t launch_sequence(const BatchParams &bp_in, int barrier_extra, bool one, cudaStream_t s) {
   if (bp_in.M != 1) return cudaErrorInvalidValue;
   thread_local BatchParams bp;
   bp = bp_in;
@@ -1650,7 +1670,10 @@ cudaError_t launch_gemv_sequence(const BatchParams &bp_in, int barrier_extra, cu
   const int gtasks = g4::stage_groups(1) * ((gmax + g4::stage_groups(1) - 1) / g4::stage_groups(1));
   const cudaError_t e = launch_prep(bp, mt, nullptr, gtasks, s);
   if (e != cudaSuccess) return e;
-  return launch_gemv_seq(bp, num_sms_mm(), barrier_extra, s);
+  return launch_gemv_seq(bp, num_sms_mm(), barrier_extra, one, s);
+}
+cudaError_t launch_gemv_sequence(const BatchParams &bp, int barrier_extra, cudaStream_t s) {
+  return launch_sequence(bp, barrier_extra, false, s);
 }
 
 cudaError_t launch_gemv_mma(const BatchParams &bp, cudaStream_t s) {

@@ -288,3 +288,31 @@ def test_split_tiles_single_call(H, M, N, K, frac, index):
         y = tq.tq_linear_f32out(x, pw, ws=ws)
         H.device_status_ok()
         H.assert_close(y.cpu().numpy().astype(np.float64), y_ref, a_ref)
+
+
+@pytest.mark.parametrize("N,K,frac", [(1, 128, 1.0), (255, 640, 0.5), (257, 1024, 0.02), (8193, 256, 0.3),
+                                      (700, 12288, 1.0)])
+@pytest.mark.parametrize("f32", [False, True])
+def test_one_token_one_indexed_weight(H, N, K, frac, f32):
+    """Both planes in one kernel: rows at the edges of tiles, of a CTA's threads
+    and of the last CTA's rounds; two calls at once on two streams, twice (its
+    counter restarts with every call)."""
+    from paper_2609_09240_gb300 import tq
+    w = wl.gen_weights(N, K, frac, config=6, proj=N)
+    x = wl.gen_x(1, K, config=6, proj=N)
+    y_ref, a_ref = H.oracle_ref(w, x)
+    pw, xd = H.pack_on_gpu(w), H.dev(x)
+    fn = tq.tq_linear_f32out if f32 else tq.tq_linear
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    ws = [tq.workspace(tq.tq_workspace_bytes(1, N, K), "cuda") for _ in streams]
+    ys = [torch.empty((1, N), dtype=torch.float32 if f32 else torch.float16, device="cuda") for _ in streams]
+    for _ in range(2):
+        for y in ys:
+            y.fill_(float("nan"))
+        torch.cuda.synchronize()
+        for st, wsp, y in zip(streams, ws, ys):
+            with torch.cuda.stream(st):
+                fn(xd, pw, y=y, ws=wsp)
+        H.device_status_ok()
+        for y in ys:
+            H.assert_close(y.float().cpu().numpy().astype(np.float64), y_ref, a_ref)
