@@ -3,6 +3,8 @@
 // kernel-side problem descriptor).
 #pragma once
 
+#include <cstddef>
+#include <cstring>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -48,7 +50,8 @@ struct Problem {
   __host__ __device__ void *map() const { return wsB + map_off; }
 };
 
-struct BatchParams {
+template <int CAP>
+struct Params {
   int32_t count;        // problems in prob[]
   int32_t M;            // tokens (rows of every x)
   int32_t total_tiles;  // sum of tiles over problems
@@ -58,8 +61,32 @@ struct BatchParams {
                         // kernel's operands are then not in the workspace)
   int32_t g4_only;      // nonzero: only the one-group-per-lane kernels read the activation operands
                         // (the prep kernel writes no general-layout fragments or C/S)
-  Problem prob[TQ_MAX_BATCH];
+  Problem prob[CAP];
 };
+using BatchParams = Params<TQ_MAX_BATCH>;
+// The launch parameters of a call of few problems: the same layout with room
+// for as many only.  31 KB of parameters cost 1.0 us more per launch than 1 KB
+// (2.6 against 1.6), and a small call is as long as its launches.
+constexpr int kFewProblems = 8;
+using FewParams = Params<kFewProblems>;
+__host__ __device__ inline const BatchParams &all_params(const BatchParams &p) { return p; }
+__host__ __device__ inline const BatchParams &all_params(const FewParams &p) {
+  return reinterpret_cast<const BatchParams &>(p);  // only prob[0 .. count) is read
+}
+// dst = src, as far as it is filled (dst has room for its problems).
+template <class BP>
+inline void copy_params(BP &dst, const BatchParams &src) {
+  std::memcpy(static_cast<void *>(&dst), static_cast<const void *>(&src),
+              offsetof(BatchParams, prob) + (size_t)src.count * sizeof(Problem));
+}
+// fn with the smallest parameters that hold bp.
+template <class Fn>
+inline cudaError_t with_params(const BatchParams &bp, Fn fn) {
+  if (bp.count > kFewProblems) return fn(bp);
+  FewParams few;
+  copy_params(few, bp);
+  return fn(few);
+}
 
 // One problem of an element-wise call as the API hands it to the kernels
 // (tq_ew.cu): the weight, x, the fp32 plane-1 result, y and the views of

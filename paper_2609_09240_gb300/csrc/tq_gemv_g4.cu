@@ -47,9 +47,11 @@
 #include <cuda.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "tq_common.cuh"
 #include "tq_decode_ops.cuh"
+#include "tq_launch.cuh"
 #include "tq_p2_tile.cuh"
 #include "tq_sm100.cuh"
 
@@ -430,9 +432,10 @@ __device__ __forceinline__ void produce_stage(unsigned char *dyn, Bars *bars, in
 
 // WD decode warps with TL m16 tiles each (WD x TL x 16 = 256 rows), and one
 // producer warp; SG groups per stage (8 for one token, 4 for two).
-template <bool F32, int MB, int SG, int WD, int TL>
+template <bool F32, int MB, int SG, int WD, int TL, class BP>
 __global__ void __launch_bounds__((WD + 1) * 32, 1)
-    gemv_g4_kernel(const __grid_constant__ BatchParams bp, const __grid_constant__ Sched sc) {
+    gemv_g4_kernel(const __grid_constant__ BP params, const __grid_constant__ Sched sc) {
+  const BatchParams &bp = all_params(params);
   using C = Cfg<SG>;
   static_assert(WD * TL * 16 == kRows && WD <= kMaxWarps, "decode warps cover the tile");
   static_assert((SG == 8 && MB == 1) || (SG == 4 && MB == 2), "stage shape per token count");
@@ -451,9 +454,8 @@ __global__ void __launch_bounds__((WD + 1) * 32, 1)
   __syncthreads();
   // everything below reads what the prep and second-plane kernels wrote
   grid_dep_wait();
-  // a programmatically launched successor (the next call's prep kernel)
-  // may be scheduled now; it waits for this grid before touching memory
-  grid_dep_launch_next();
+  // (the next call's prep kernel is let in only when this one ends: its blocks
+  // waiting beside these took the Qwen3-8B step from 492 us to 508)
   const int t_begin = sc.cta_unit[blockIdx.x], t_end = sc.cta_unit[blockIdx.x + 1];
 
   if (warp < WD) {
@@ -716,7 +718,9 @@ __device__ __forceinline__ void prefetch_second_plane(const Problem &P, int cta,
 // (a ticket from the counter) stores all of y.
 template <bool F32, bool ONE>
 __global__ void __launch_bounds__((kWD1 + 1 + kSeqP2) * 32, 1)
-    gemv_seq_kernel(const __grid_constant__ BatchParams bp, int32_t barrier_extra) {
+    gemv_seq_kernel(const __grid_constant__ std::conditional_t<ONE, FewParams, BatchParams> params,
+                    int32_t barrier_extra) {
+  const BatchParams &bp = all_params(params);
   constexpr int SG = 8, MB = 1, WD = kWD1, TL = kTL1;
   using C = Cfg<SG>;
   constexpr int kNS = C::kNS;
@@ -939,8 +943,10 @@ __host__ __device__ inline int p2r_parts(int K, int64_t nnz, int tiles) {
   return (int)(q < 1 ? 1 : q > 64 ? 64 : q);
 }
 
+template <class BP>
 __global__ void __launch_bounds__(kP2rWarps * 32, 1)
-    gemv_p2r_kernel(const __grid_constant__ P2rBase pb, const __grid_constant__ BatchParams bp, int32_t *counter) {
+    gemv_p2r_kernel(const __grid_constant__ P2rBase pb, const __grid_constant__ BP params, int32_t *counter) {
+  const BatchParams &bp = all_params(params);
   extern __shared__ __align__(1024) unsigned char dynr[];
   const int tid = threadIdx.x, lane = tid & 31;
   if (smem_u32(dynr) != kDynShared) {
@@ -1136,24 +1142,16 @@ cudaError_t launch_gemv_g4(const BatchParams &bp, int num_sms, cudaStream_t s) {
   using g4::kTL2;
   using g4::kWD1;
   using g4::kWD2;
-  auto kern = bp.M == 1
-                  ? (bp.out_f32 ? g4::gemv_g4_kernel<true, 1, 8, kWD1, kTL1> : g4::gemv_g4_kernel<false, 1, 8, kWD1, kTL1>)
-                  : (bp.out_f32 ? g4::gemv_g4_kernel<true, 2, 4, kWD2, kTL2> : g4::gemv_g4_kernel<false, 2, 4, kWD2, kTL2>);
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, g4::kDynBytes);
-  if (e != cudaSuccess) return e;
   // launched programmatically: its CTAs set up (table, barriers) while the
   // second-plane kernel finishes, then wait for it (grid_dep_wait)
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(ctas);
-  cfg.blockDim = dim3(((bp.M == 1 ? kWD1 : kWD2) + 1) * 32);
-  cfg.dynamicSmemBytes = g4::kDynBytes;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, bp, sc);
+  return with_params(bp, [&](const auto &p) {
+    using BP = std::decay_t<decltype(p)>;
+    auto kern = bp.M == 1 ? (bp.out_f32 ? g4::gemv_g4_kernel<true, 1, 8, kWD1, kTL1, BP>
+                                        : g4::gemv_g4_kernel<false, 1, 8, kWD1, kTL1, BP>)
+                          : (bp.out_f32 ? g4::gemv_g4_kernel<true, 2, 4, kWD2, kTL2, BP>
+                                        : g4::gemv_g4_kernel<false, 2, 4, kWD2, kTL2, BP>);
+    return launch_big_smem(kern, ctas, ((bp.M == 1 ? kWD1 : kWD2) + 1) * 32, g4::kDynBytes, s, p, sc);
+  });
 }
 
 // The second plane of one token through gemv_p2r_kernel (every problem
@@ -1176,19 +1174,10 @@ cudaError_t launch_gemv_p2r(const BatchParams &bp, int num_sms, int32_t *counter
     const Problem &P = bp.prob[p];
     pb.base[p + 1] = pb.base[p] + (P.nnz > 0 ? g4::nstages(P.K, 8) * g4::p2r_parts(P.K, P.nnz, pb.tiles) : 0);
   }
-  cudaError_t e = cudaFuncSetAttribute(g4::gemv_p2r_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, g4::kP2rDyn);
-  if (e != cudaSuccess) return e;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(ctas);
-  cfg.blockDim = dim3(g4::kP2rWarps * 32);
-  cfg.dynamicSmemBytes = g4::kP2rDyn;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, g4::gemv_p2r_kernel, pb, bp, counter);
+  return with_params(bp, [&](const auto &p) {
+    return launch_big_smem(g4::gemv_p2r_kernel<std::decay_t<decltype(p)>>, ctas, g4::kP2rWarps * 32, g4::kP2rDyn, s, pb,
+                           p, counter);
+  });
 }
 
 // The dependency-ordered sequence kernel (one token), launched
@@ -1197,21 +1186,14 @@ cudaError_t launch_gemv_p2r(const BatchParams &bp, int num_sms, int32_t *counter
 cudaError_t launch_gemv_seq(const BatchParams &bp, int num_sms, int barrier_extra, bool one, cudaStream_t s) {
   if (bp.M != 1 || bp.count < 1 || (one && bp.count != 1)) return cudaErrorInvalidValue;
   const int ctas = std::min(num_sms, 256);
-  auto kern = one ? (bp.out_f32 ? g4::gemv_seq_kernel<true, true> : g4::gemv_seq_kernel<false, true>)
-                  : (bp.out_f32 ? g4::gemv_seq_kernel<true, false> : g4::gemv_seq_kernel<false, false>);
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, g4::kDynBytes);
-  if (e != cudaSuccess) return e;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(ctas);
-  cfg.blockDim = dim3((g4::kWD1 + 1 + g4::kSeqP2) * 32);
-  cfg.dynamicSmemBytes = g4::kDynBytes;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, bp, (int32_t)barrier_extra);
+  constexpr int threads = (g4::kWD1 + 1 + g4::kSeqP2) * 32;
+  if (!one)
+    return launch_big_smem(bp.out_f32 ? g4::gemv_seq_kernel<true, false> : g4::gemv_seq_kernel<false, false>, ctas, threads,
+                           g4::kDynBytes, s, bp, (int32_t)barrier_extra);
+  FewParams few;
+  copy_params(few, bp);
+  return launch_big_smem(bp.out_f32 ? g4::gemv_seq_kernel<true, true> : g4::gemv_seq_kernel<false, true>, ctas, threads,
+                         g4::kDynBytes, s, few, (int32_t)barrier_extra);
 }
 
 }  // namespace tq

@@ -316,3 +316,21 @@ def test_one_token_one_indexed_weight(H, N, K, frac, f32):
         H.device_status_ok()
         for y in ys:
             H.assert_close(y.float().cpu().numpy().astype(np.float64), y_ref, a_ref)
+
+
+@pytest.mark.parametrize("count", [8, 9])
+@pytest.mark.parametrize("M,index", [(1, True), (1, False), (2, True), (5, False), (12, True)])
+def test_batched_parameter_sizes(H, count, M, index):
+    """The most problems that fit the small launch parameters, and one more."""
+    from paper_2609_09240_gb300 import tq
+    items, refs = [], []
+    for i in range(count):
+        N, K = 100 + 37 * i, 128 * (1 + i % 4)
+        w = wl.gen_weights(N, K, 0.2, config=6, proj=i)
+        x = wl.gen_x(M, K, config=6, proj=i)
+        refs.append(H.oracle_ref(w, x))
+        items.append((H.pack_on_gpu(w, index=index), H.dev(x), torch.empty((M, N), dtype=torch.float16, device="cuda")))
+    tq.tq_linear_batched(tq.Batch(M, items))
+    H.device_status_ok()
+    for (_, _, y), (y_ref, a_ref) in zip(items, refs):
+        H.assert_close(y.float().cpu().numpy().astype(np.float64), y_ref, a_ref)
