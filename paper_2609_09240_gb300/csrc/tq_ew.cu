@@ -15,6 +15,8 @@
 #include <algorithm>
 
 #include "tq_common.cuh"
+#include "tq_launch.cuh"
+#include "tq_sm100.cuh"
 
 namespace tq {
 namespace ew {
@@ -43,7 +45,7 @@ struct Prob {
   const float *ydense;         // [M][N]
   void *y;                     // [M][N], fp16 or fp32
   int32_t N, K, S, blocks;     // blocks = 0: the problem is the other kernel's
-  int32_t row_begin;           // first row of the problem among the index kernel's rows
+  int64_t w_begin;             // N G of the index kernel's problems before it
 };
 template <typename T>
 struct Batch {
@@ -260,83 +262,179 @@ __global__ void __launch_bounds__(32 * kWarps) correct_kernel(const __grid_const
 }
 
 constexpr int kIdxBlock = 2048, kIdxShift = 11;  // the correction index's blocks and code position
-constexpr uint32_t kIdxNone = 31u << kIdxShift;  // a code that weighs nothing (pads a step)
+constexpr int kIdxWarps = 16, kIdxThreads = 32 * kIdxWarps;
+constexpr int kIdxAhead = 8;  // entries per lane loaded one block ahead
+constexpr int kIdxTabBytes = kIdxWarps * 32 * 4;
+constexpr int kIdxMaxSmem = 227 * 1024, kSmSmem = 228 * 1024;  // shared memory of a block, of an SM
 
-// The same correction from the correction index: warp per row, the warps
-// striding over the rows of every indexed problem of the call; the lanes
-// take a block's entries two at a time per step.  An entry names its element
-// k (within its block) and code = 9 q + 3 d0 + d1 (digits d = trit + 1),
-// whose weight (mu_q - mu_3) + (alpha0_q - alpha0_3) T0 + alpha1_q T1 is read
-// from the row's 27-entry table.  Only the entries and x are read: no mask
-// plane, plane-1 or plane-2 bytes.
-template <bool F32, int MT>
-__global__ void __launch_bounds__(32 * kWarps) correct_idx_kernel(const __grid_constant__ Batch<Prob> bt,
-                                                                  int total_rows, int m0, int mt) {
-  __shared__ float tab[kWarps][32];
+// Bytes of correct_idx_kernel's staged activations: MT fp16 per element,
+// whole blocks.
+__host__ __device__ constexpr int64_t stage_bytes(int K, int MT) {
+  return (int64_t)((K + kIdxBlock - 1) / kIdxBlock) * kIdxBlock * MT * 2;
+}
+
+// MT activations of one element, fp16, side by side.
+template <int MT>
+struct Acts;
+template <>
+struct Acts<1> {
+  unsigned short h[1];
+};
+template <>
+struct alignas(4) Acts<2> {
+  unsigned short h[2];
+};
+template <>
+struct alignas(8) Acts<4> {
+  unsigned short h[4];
+};
+template <>
+struct alignas(16) Acts<8> {
+  unsigned short h[8];
+};
+
+// The same correction from the correction index.  An entry names its element
+// k (within its block of 2048) and code = 9 q + 3 d0 + d1 (digits d = trit +
+// 1), whose weight (mu_q - mu_3) + (alpha0_q - alpha0_3) T0 + alpha1_q T1 is
+// read from the row's 27-entry table.  Only the entries and x are read: no
+// mask plane, plane-1 or plane-2 bytes.
+//
+// The rows of every indexed problem of the call, one after the other and
+// weighted with their length, are cut into one run per block; a block's
+// warps take the run's rows in turn.  The kernel is bound by its gathers of x: from
+// global memory a warp's 32 lanes touch some 20 cache lines per load (48 us
+// for the 27 M entries of one Qwen3-8B layer), from shared memory the same
+// 32 words cost three to four bank cycles.  So a block stages x[tokens][K],
+// the tokens of an element side by side, whenever its run enters another
+// problem (24 KB for K = 12288, against 121 rows of 3.3 KB of entries), and
+// the lanes load a block's entries (eight each, what 13.6 % coverage has,
+// the rest in a loop) while they work on the block before.  A batched layer
+// call (Qwen3-8B) takes 78.9 us with it for one token (86.7 with gathers from
+// global memory), 84.5 (103.1) for two, 90.1 (136.3) for four and 204 (404)
+// for sixteen.  STAGED = false reads x from global memory: K x tokens beyond
+// a block's shared memory.
+template <bool F32, int MT, bool STAGED>
+__global__ void __launch_bounds__(kIdxThreads, MT == 8 ? 1 : 2)
+    correct_idx_kernel(const __grid_constant__ Batch<Prob> bt, int64_t total, int m0, int mt) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  float *tab = reinterpret_cast<float *>(smem) + (threadIdx.x >> 5) * 32;
+  Acts<MT> *xs = reinterpret_cast<Acts<MT> *>(smem + kIdxTabBytes);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int top = 1 << (31 - __clz(max(bt.count, 1)));
-  for (int r = blockIdx.x * kWarps + warp; r < total_rows; r += gridDim.x * kWarps) {
-    // the problem of row r: the last with row_begin <= r (problems without
-    // an index have no rows: their row_begin equals the next one's)
-    int p = 0;
-    for (int step = top; step >= 1; step >>= 1)
-      if (p + step < bt.count && bt.prob[p + step].row_begin <= r) p += step;
+  // the block's run: row r of problem p lies in it if its first weight unit
+  // (w_begin + r G) does
+  const int64_t u_lo = total * blockIdx.x / gridDim.x, u_hi = total * (blockIdx.x + 1) / gridDim.x;
+  int p = 0;
+  for (int step = 1 << (31 - __clz(max(bt.count, 1))); step >= 1; step >>= 1)
+    if (p + step < bt.count && bt.prob[p + step].w_begin <= u_lo) p += step;
+  bool waited = false;
+  for (; p < bt.count; ++p) {
     const Prob &w = bt.prob[p];
-    const int n = r - w.row_begin, N = w.N, K = w.K;
-    {
-      // codes 27..31 (none in a valid index but the step padding) weigh nothing
-      const int q = lane / 9, d0 = (lane / 3) % 3, d1 = lane % 3;
-      float v = 0.f;
-      if (lane < 27) {
-        const __half *mu = w.mu + (int64_t)n * 4, *a0 = w.a0 + (int64_t)n * 4;
-        v = (__half2float(mu[q]) - __half2float(mu[3])) + (__half2float(a0[q]) - __half2float(a0[3])) * (float)(d0 - 1);
-        if (q < 2) v += __half2float(w.a1[(int64_t)n * 2 + q]) * (float)(d1 - 1);
-      }
-      tab[warp][lane] = v;
-    }
-    __syncwarp();
-    const float *tw = tab[warp];
-    const uint16_t *idx = w.idx;
+    if (w.w_begin >= u_hi) break;
+    if (!w.idx) continue;  // the other kernel's
+    const int N = w.N, K = w.K, G = K / kGroup;
+    const int r_lo = (int)min((int64_t)N, (max(u_lo - w.w_begin, (int64_t)0) + G - 1) / G);
+    const int r_hi = (int)min((int64_t)N, (u_hi - w.w_begin + G - 1) / G);
+    if (r_lo >= r_hi) continue;
     const unsigned short *xm = reinterpret_cast<const unsigned short *>(w.x) + (int64_t)m0 * K;
-    const int nb = (K + kIdxBlock - 1) / kIdxBlock;
-    const int32_t *offr = w.idx_off + (int64_t)n * nb;
-    float acc[MT];
-#pragma unroll
-    for (int t = 0; t < MT; ++t) acc[t] = 0.f;
-    int e = __ldg(offr);
-    for (int b = 0; b < nb; ++b) {
-      const int e1 = __ldg(offr + b + 1);
-      const int kb = b * kIdxBlock, kmax = K - 1 - kb;
-      for (int e0 = e + lane; e0 < e1; e0 += 64) {
-        const uint32_t v0 = __ldg(idx + e0);
-        const uint32_t v1 = e0 + 32 < e1 ? __ldg(idx + e0 + 32) : kIdxNone;
-        const int k0 = kb + min((int)(v0 & (kIdxBlock - 1)), kmax), k1 = kb + min((int)(v1 & (kIdxBlock - 1)), kmax);
-        const float w0 = tw[v0 >> kIdxShift], w1 = tw[v1 >> kIdxShift];
+    if (STAGED) {
+      __syncthreads();  // the warps are done with the problem before
+      for (int i = threadIdx.x; i < K / 8; i += kIdxThreads) {
+        uint4 v[MT];
 #pragma unroll
         for (int t = 0; t < MT; ++t)
-          if (t < mt) {
-            const float x0 = __half2float(__ushort_as_half(__ldg(xm + t * K + k0)));
-            const float x1 = __half2float(__ushort_as_half(__ldg(xm + t * K + k1)));
-            acc[t] = fmaf(w0, x0, fmaf(w1, x1, acc[t]));
+          v[t] = t < mt ? __ldg(reinterpret_cast<const uint4 *>(xm + (int64_t)t * K) + i) : make_uint4(0u, 0u, 0u, 0u);
+        if (MT == 1) {
+          reinterpret_cast<uint4 *>(xs)[i] = v[0];
+        } else {
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            Acts<MT> a;
+#pragma unroll
+            for (int t = 0; t < MT; ++t) {
+              const uint32_t word = (j >> 1) == 0 ? v[t].x : (j >> 1) == 1 ? v[t].y : (j >> 1) == 2 ? v[t].z : v[t].w;
+              a.h[t] = (unsigned short)(j & 1 ? word >> 16 : word & 0xffffu);
+            }
+            xs[8 * i + j] = a;
           }
+        }
       }
-      e = e1;
+      __syncthreads();
     }
+    const uint16_t *idx = w.idx;
+    const int nb = (K + kIdxBlock - 1) / kIdxBlock;
+    for (int n = r_lo + warp; n < r_hi; n += kIdxWarps) {
+      const int32_t *offr = w.idx_off + (int64_t)n * nb;
+      int e = __ldg(offr), e1 = __ldg(offr + 1);
+      uint32_t v[kIdxAhead];
 #pragma unroll
-    for (int t = 0; t < MT; ++t) {
-      float v = acc[t];
+      for (int j = 0; j < kIdxAhead; ++j) v[j] = e + lane + 32 * j < e1 ? __ldg(idx + e + lane + 32 * j) : 0u;
+      __syncwarp();  // the row before is done with the table
+      {
+        // codes 27..31 (none in a valid index) weigh nothing
+        const int q = lane / 9, d0 = (lane / 3) % 3, d1 = lane % 3;
+        float a = 0.f;
+        if (lane < 27) {
+          const __half *mu = w.mu + (int64_t)n * 4, *a0 = w.a0 + (int64_t)n * 4;
+          a = (__half2float(mu[q]) - __half2float(mu[3])) +
+              (__half2float(a0[q]) - __half2float(a0[3])) * (float)(d0 - 1);
+          if (q < 2) a += __half2float(w.a1[(int64_t)n * 2 + q]) * (float)(d1 - 1);
+        }
+        tab[lane] = a;
+      }
+      __syncwarp();
+      float acc[MT];
 #pragma unroll
-      for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-      if (lane == t && t < mt) {
-        const int64_t i = (int64_t)(m0 + t) * N + n;
-        v += w.ydense[i];
+      for (int t = 0; t < MT; ++t) acc[t] = 0.f;
+      for (int b = 0; b < nb; ++b) {
+        const int e2 = b + 1 < nb ? __ldg(offr + b + 2) : e1;
+        uint32_t u[kIdxAhead];  // the next block's entries
+#pragma unroll
+        for (int j = 0; j < kIdxAhead; ++j) u[j] = e1 + lane + 32 * j < e2 ? __ldg(idx + e1 + lane + 32 * j) : 0u;
+        const int kb = b * kIdxBlock, kmax = K - 1 - kb;
+        auto add = [&](uint32_t en) {
+          const int k = kb + min((int)(en & (kIdxBlock - 1)), kmax);
+          const float wt = tab[en >> kIdxShift];
+          if (STAGED) {
+            const Acts<MT> a = xs[k];
+#pragma unroll
+            for (int t = 0; t < MT; ++t) acc[t] = fmaf(wt, __half2float(__ushort_as_half(a.h[t])), acc[t]);
+          } else {
+#pragma unroll
+            for (int t = 0; t < MT; ++t)
+              if (t < mt) acc[t] = fmaf(wt, __half2float(__ushort_as_half(__ldg(xm + (int64_t)t * K + k))), acc[t]);
+          }
+        };
+        const int c = e1 - e;
+#pragma unroll
+        for (int j = 0; j < kIdxAhead; ++j) {
+          if (32 * j >= c) break;
+          if (lane + 32 * j < c) add(v[j]);
+        }
+        for (int e0 = e + lane + 32 * kIdxAhead; e0 < e1; e0 += 32) add(__ldg(idx + e0));
+        e = e1;
+        e1 = e2;
+#pragma unroll
+        for (int j = 0; j < kIdxAhead; ++j) v[j] = u[j];
+      }
+      float mine = 0.f;
+#pragma unroll
+      for (int t = 0; t < MT; ++t) {
+        float s = acc[t];
+#pragma unroll
+        for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (lane == t) mine = s;
+      }
+      if (!waited) grid_dep_wait();  // the plane-1 pass; what stands above reads only the caller's arrays
+      waited = true;
+      if (lane < mt && lane < MT) {
+        const int64_t i = (int64_t)(m0 + lane) * N + n;
+        mine += w.ydense[i];
         if (F32)
-          static_cast<float *>(w.y)[i] = v;
+          static_cast<float *>(w.y)[i] = mine;
         else
-          static_cast<__half *>(w.y)[i] = __float2half_rn(v);
+          static_cast<__half *>(w.y)[i] = __float2half_rn(mine);
       }
     }
-    __syncwarp();  // the table is rewritten for the next row
   }
 }
 
@@ -351,26 +449,55 @@ int warps_per_row(int N, int K, int num_sms) {
   return S;
 }
 
-// indexed: grid blocks striding over `rows` rows; else grid x count.
 template <bool F32, int MT>
-cudaError_t launch_correct(int M, const Batch<Prob> &bt, int grid, int rows, bool indexed, cudaStream_t s) {
+cudaError_t launch_correct(int M, const Batch<Prob> &bt, int grid, cudaStream_t s) {
   for (int m0 = 0; m0 < M; m0 += MT) {
-    if (indexed)
-      correct_idx_kernel<F32, MT><<<grid, 32 * kWarps, 0, s>>>(bt, rows, m0, std::min(MT, M - m0));
-    else
-      correct_kernel<F32, MT><<<dim3(grid, bt.count), 32 * kWarps, 0, s>>>(bt, m0, std::min(MT, M - m0));
+    correct_kernel<F32, MT><<<dim3(grid, bt.count), 32 * kWarps, 0, s>>>(bt, m0, std::min(MT, M - m0));
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
 }
 
+// grid: blocks for the call's indexed rows at one row per warp, capped at
+// what the chip holds.
+template <bool F32, int MT, bool STAGED>
+cudaError_t launch_correct_idx(int M, const Batch<Prob> &bt, int64_t total, int rows, int Kmax, int num_sms,
+                               cudaStream_t s) {
+  const int smem = kIdxTabBytes + (STAGED ? (int)stage_bytes(Kmax, MT) : 0);
+  const auto kern = correct_idx_kernel<F32, MT, STAGED>;
+  const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kIdxMaxSmem);
+  if (e != cudaSuccess) return e;
+  const int per_sm = MT < 8 && 2 * (smem + 1024) <= kSmSmem ? 2 : 1;
+  const int grid = std::max(1, std::min((rows + kIdxWarps - 1) / kIdxWarps, per_sm * num_sms));
+  for (int m0 = 0; m0 < M; m0 += MT) {
+    const cudaError_t l =
+        launch_dependent_cluster(kern, dim3(grid), 1, kIdxThreads, smem, s, bt, total, m0, std::min(MT, M - m0));
+    if (l != cudaSuccess) return l;
+  }
+  return cudaSuccess;
+}
+
 template <bool F32>
-cudaError_t launch_correct_mt(int M, const Batch<Prob> &bt, int grid, int rows, bool indexed, cudaStream_t s) {
-  if (M == 1) return launch_correct<F32, 1>(M, bt, grid, rows, indexed, s);
-  if (M == 2) return launch_correct<F32, 2>(M, bt, grid, rows, indexed, s);
-  if (M <= 4) return launch_correct<F32, 4>(M, bt, grid, rows, indexed, s);
-  return launch_correct<F32, 8>(M, bt, grid, rows, indexed, s);
+cudaError_t launch_correct_mt(int M, const Batch<Prob> &bt, int grid, cudaStream_t s) {
+  if (M == 1) return launch_correct<F32, 1>(M, bt, grid, s);
+  if (M == 2) return launch_correct<F32, 2>(M, bt, grid, s);
+  if (M <= 4) return launch_correct<F32, 4>(M, bt, grid, s);
+  return launch_correct<F32, 8>(M, bt, grid, s);
+}
+
+// Tokens per pass: as many as the call has, up to 8, while their staged
+// activations fit a block's shared memory (K up to 14336 for 8 tokens,
+// 114688 for one); beyond that x is gathered from global memory.
+template <bool F32>
+cudaError_t launch_correct_idx_mt(int M, const Batch<Prob> &bt, int64_t total, int rows, int Kmax, int num_sms,
+                                  cudaStream_t s) {
+  const auto fits = [&](int MT) { return kIdxTabBytes + stage_bytes(Kmax, MT) <= kIdxMaxSmem; };
+  if (M > 4 && fits(8)) return launch_correct_idx<F32, 8, true>(M, bt, total, rows, Kmax, num_sms, s);
+  if (M > 2 && fits(4)) return launch_correct_idx<F32, 4, true>(M, bt, total, rows, Kmax, num_sms, s);
+  if (M > 1 && fits(2)) return launch_correct_idx<F32, 2, true>(M, bt, total, rows, Kmax, num_sms, s);
+  if (M == 1 && fits(1)) return launch_correct_idx<F32, 1, true>(M, bt, total, rows, Kmax, num_sms, s);
+  return launch_correct_idx<F32, 8, false>(M, bt, total, rows, Kmax, num_sms, s);
 }
 
 }  // namespace ew
@@ -410,7 +537,8 @@ cudaError_t launch_ew_correct(int M, const EwCall *calls, int count, bool f32, c
   bt.count = count;
   for (int pass = 0; pass < 2; ++pass) {
     const bool indexed = pass == 1;
-    int most = 0, total = 0;
+    int most = 0, rows_idx = 0, Kmax = 0;
+    int64_t total = 0;
     for (int i = 0; i < count; ++i) {
       const EwCall &c = calls[i];
       ew::Prob &P = bt.prob[i];
@@ -432,14 +560,19 @@ cudaError_t launch_ew_correct(int M, const EwCall *calls, int count, bool f32, c
       P.S = ew::warps_per_row(P.N, P.K, sms);
       const int rows = ew::kWarps / P.S;
       P.blocks = mine && !indexed ? (P.N + rows - 1) / rows : 0;
-      P.row_begin = total;
-      if (mine && indexed) total += P.N;
+      P.w_begin = total;
+      if (mine && indexed) {
+        total += (int64_t)P.N * (P.K / kGroup);
+        rows_idx = std::min<int64_t>((int64_t)rows_idx + P.N, INT32_MAX / 2);
+        Kmax = std::max(Kmax, P.K);
+      }
       most = std::max(most, P.blocks);
     }
     if (indexed ? total == 0 : most == 0) continue;
-    const int grid = indexed ? std::min((total + ew::kWarps - 1) / ew::kWarps, 8 * sms) : most;
-    const cudaError_t e = f32 ? ew::launch_correct_mt<true>(M, bt, grid, total, indexed, s)
-                              : ew::launch_correct_mt<false>(M, bt, grid, total, indexed, s);
+    const cudaError_t e = indexed ? (f32 ? ew::launch_correct_idx_mt<true>(M, bt, total, rows_idx, Kmax, sms, s)
+                                         : ew::launch_correct_idx_mt<false>(M, bt, total, rows_idx, Kmax, sms, s))
+                                  : (f32 ? ew::launch_correct_mt<true>(M, bt, most, s)
+                                         : ew::launch_correct_mt<false>(M, bt, most, s));
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;

@@ -260,3 +260,25 @@ def test_linear_indexed_qwen3_8b_shapes_sampled_rows(H, N, K):
     y = tq.tq_ew_linear(H.dev(xb), _indexed(H, w))
     H.device_status_ok()
     H.assert_close(y.float().cpu().numpy()[:, rows].astype(np.float64), y_ref, a_ref)
+
+
+@pytest.mark.parametrize("M,N,K,cover", [
+    (1, 5000, 384, (0.3, 0.3, 0.4)),        # every element indexed, runs that begin inside a problem
+    (4, 33, 2176, (0.4, 0.3, 0.3)),         # blocks of 2048 entries: more than a warp loads ahead; a last block of 128
+    (1, 40, 4096, (0.0, 0.0, 0.0)),         # empty rows
+    (3, 17, 32768, (0.005, 0.031, 0.10)),   # x of four tokens exceeds a block's shared memory: passes of two
+    (16, 19, 16384, (0.005, 0.031, 0.10)),  # passes of four
+    (1, 3, 131072, (0.005, 0.031, 0.10)),   # x from global memory
+    (5, 3, 131072, (0.005, 0.031, 0.10)),
+])
+def test_linear_indexed_runs_and_staging(H, M, N, K, cover):
+    from paper_2609_09240_gb300 import tq
+    w = wl.gen_ew_weights(N, K, config=25, proj=M + N, coverage=cover)
+    xb = wl.gen_x(M, K, config=25, proj=M + N)
+    mp, p1, rp, p2, st = ew.pack(w.T0, w.T1, w.mask)
+    assert st == 0
+    rows = np.arange(N) if N <= 64 else np.sort(np.random.default_rng(N).choice(N, size=200, replace=False))
+    y_ref, a_ref = ew.linear(xb, K, mp, p1, rp, p2, w.mu, w.a0, w.a1, rows=rows)
+    y = tq.tq_ew_linear(H.dev(xb), _indexed(H, w))
+    H.device_status_ok()
+    H.assert_close(y.float().cpu().numpy()[:, rows].astype(np.float64), y_ref, a_ref)
