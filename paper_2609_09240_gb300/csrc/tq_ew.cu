@@ -263,35 +263,45 @@ __global__ void __launch_bounds__(32 * kWarps) correct_kernel(const __grid_const
 
 constexpr int kIdxBlock = 2048, kIdxShift = 11;  // the correction index's blocks and code position
 constexpr int kIdxWarps = 16, kIdxThreads = 32 * kIdxWarps;
-constexpr int kIdxAhead = 8;  // entries per lane loaded one block ahead
+constexpr int kIdxAhead = 5;  // pairs of entries per lane loaded one block ahead
 constexpr int kIdxTabBytes = kIdxWarps * 32 * 4;
 constexpr int kIdxMaxSmem = 227 * 1024, kSmSmem = 228 * 1024;  // shared memory of a block, of an SM
 
-// Bytes of correct_idx_kernel's staged activations: MT fp16 per element,
-// whole blocks.
-__host__ __device__ constexpr int64_t stage_bytes(int K, int MT) {
-  return (int64_t)((K + kIdxBlock - 1) / kIdxBlock) * kIdxBlock * MT * 2;
+// Staged bytes per element: one token as fp32, more side by side as fp16.
+__host__ __device__ constexpr int elem_bytes(int MT) { return MT == 1 ? 4 : 2 * MT; }
+// correct_idx_kernel's dynamic shared memory: the warps' tables, then the
+// activations from the next multiple of a block's bytes on.
+constexpr int64_t idx_smem_bytes(int K, int MT) {
+  return (int64_t)((K + kIdxBlock - 1) / kIdxBlock + 1) * kIdxBlock * elem_bytes(MT);
 }
 
-// MT activations of one element, fp16, side by side.
+__device__ __forceinline__ float half_at(uint32_t w, int hi) {
+  return __half2float(__ushort_as_half((unsigned short)(hi ? w >> 16 : w & 0xffffu)));
+}
+__device__ __forceinline__ float lds_f32(uint32_t a) {
+  float v;
+  asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a));
+  return v;
+}
+// The MT activations of the element staged at shared address a.
 template <int MT>
-struct Acts;
-template <>
-struct Acts<1> {
-  unsigned short h[1];
-};
-template <>
-struct alignas(4) Acts<2> {
-  unsigned short h[2];
-};
-template <>
-struct alignas(8) Acts<4> {
-  unsigned short h[4];
-};
-template <>
-struct alignas(16) Acts<8> {
-  unsigned short h[8];
-};
+__device__ __forceinline__ void staged_acts(uint32_t a, float (&x)[MT]) {
+  if constexpr (MT == 1) {
+    x[0] = lds_f32(a);
+  } else {
+    uint32_t w[MT / 2];
+    if constexpr (MT == 2)
+      asm volatile("ld.shared.u32 %0, [%1];" : "=r"(w[0]) : "r"(a));
+    else if constexpr (MT == 4)
+      asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(w[0]), "=r"(w[1]) : "r"(a));
+    else
+      asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+                   : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3])
+                   : "r"(a));
+#pragma unroll
+    for (int t = 0; t < MT; ++t) x[t] = half_at(w[t / 2], t & 1);
+  }
+}
 
 // The same correction from the correction index.  An entry names its element
 // k (within its block of 2048) and code = 9 q + 3 d0 + d1 (digits d = trit +
@@ -300,119 +310,159 @@ struct alignas(16) Acts<8> {
 // mask plane, plane-1 or plane-2 bytes.
 //
 // The rows of every indexed problem of the call, one after the other and
-// weighted with their length, are cut into one run per block; a block's
-// warps take the run's rows in turn.  The kernel is bound by its gathers of x: from
-// global memory a warp's 32 lanes touch some 20 cache lines per load (48 us
-// for the 27 M entries of one Qwen3-8B layer), from shared memory the same
-// 32 words cost three to four bank cycles.  So a block stages x[tokens][K],
-// the tokens of an element side by side, whenever its run enters another
-// problem (24 KB for K = 12288, against 121 rows of 3.3 KB of entries), and
-// the lanes load a block's entries (eight each, what 13.6 % coverage has,
-// the rest in a loop) while they work on the block before.  A batched layer
-// call (Qwen3-8B) takes 78.9 us with it for one token (86.7 with gathers from
-// global memory), 84.5 (103.1) for two, 90.1 (136.3) for four and 204 (404)
-// for sixteen.  STAGED = false reads x from global memory: K x tokens beyond
-// a block's shared memory.
+// weighted with their length, are cut into one run per block, and the block's
+// rows of a problem into one run per warp.  A block stages x[tokens][K]
+// whenever its run enters another problem, the tokens of an element side by
+// side: a gather from global memory touches some 20 cache lines per warp
+// load, the same 32 words of shared memory take three to four bank cycles.
+// Entries, offsets, table values and the plane-1 result are loaded ahead of
+// their use (the rows of a warp are contiguous, and so are their entries):
+// a lane has its ten entries of the next block (320 per warp; 13.6 % coverage
+// has 279) in registers while it works on this one; fuller blocks finish
+// in a loop.  What binds is the instructions per entry, so entries come in pairs, a table
+// or activation address is one shift and one three-input AND-OR (tables and
+// blocks lie at multiples of their size), one token is staged as fp32, and
+// entries past a block's end are cut by predicates: 20
+// warp-instructions per 32 entries with all that surrounds them, 18.4 M for
+// one Qwen3-8B layer in 28.3 us (66 % of the issue slots; 54 MB, whose floor
+// is 8 us), against 31.6 M in 39.5 us with one guarded entry per lane and
+// step, and 48 us with gathers from global memory.
+// STAGED = false reads x from global memory: K x tokens beyond a block's
+// shared memory.
 template <bool F32, int MT, bool STAGED>
 __global__ void __launch_bounds__(kIdxThreads, MT == 8 ? 1 : 2)
     correct_idx_kernel(const __grid_constant__ Batch<Prob> bt, int64_t total, int m0, int mt) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  float *tab = reinterpret_cast<float *>(smem) + (threadIdx.x >> 5) * 32;
-  Acts<MT> *xs = reinterpret_cast<Acts<MT> *>(smem + kIdxTabBytes);
+  constexpr int kES = elem_bytes(MT), kBlockBytes = kIdxBlock * kES;
+  constexpr int kESLog = MT == 8 ? 4 : MT == 4 ? 3 : 2;
+  extern __shared__ __align__(1024) unsigned char smem[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint32_t base = smem_u32(smem);
+  float *tab = reinterpret_cast<float *>(smem) + warp * 32;
+  const uint32_t tab_a = base + (uint32_t)warp * 128u;
+  const uint32_t xs_a = (base + kIdxTabBytes + kBlockBytes - 1) / kBlockBytes * kBlockBytes;
+  unsigned char *xs = smem + (xs_a - base);
   // the block's run: row r of problem p lies in it if its first weight unit
   // (w_begin + r G) does
   const int64_t u_lo = total * blockIdx.x / gridDim.x, u_hi = total * (blockIdx.x + 1) / gridDim.x;
   int p = 0;
   for (int step = 1 << (31 - __clz(max(bt.count, 1))); step >= 1; step >>= 1)
     if (p + step < bt.count && bt.prob[p + step].w_begin <= u_lo) p += step;
-  bool waited = false;
   for (; p < bt.count; ++p) {
     const Prob &w = bt.prob[p];
     if (w.w_begin >= u_hi) break;
     if (!w.idx) continue;  // the other kernel's
     const int N = w.N, K = w.K, G = K / kGroup;
-    const int r_lo = (int)min((int64_t)N, (max(u_lo - w.w_begin, (int64_t)0) + G - 1) / G);
-    const int r_hi = (int)min((int64_t)N, (u_hi - w.w_begin + G - 1) / G);
-    if (r_lo >= r_hi) continue;
+    const int b_lo = (int)min((int64_t)N, (max(u_lo - w.w_begin, (int64_t)0) + G - 1) / G);
+    const int b_hi = (int)min((int64_t)N, (u_hi - w.w_begin + G - 1) / G);
+    if (b_lo >= b_hi) continue;
     const unsigned short *xm = reinterpret_cast<const unsigned short *>(w.x) + (int64_t)m0 * K;
+    const int nb = (K + kIdxBlock - 1) / kIdxBlock;
     if (STAGED) {
       __syncthreads();  // the warps are done with the problem before
-      for (int i = threadIdx.x; i < K / 8; i += kIdxThreads) {
+      for (int i = threadIdx.x; i < nb * (kIdxBlock / 8); i += kIdxThreads) {
         uint4 v[MT];
 #pragma unroll
-        for (int t = 0; t < MT; ++t)
-          v[t] = t < mt ? __ldg(reinterpret_cast<const uint4 *>(xm + (int64_t)t * K) + i) : make_uint4(0u, 0u, 0u, 0u);
-        if (MT == 1) {
-          reinterpret_cast<uint4 *>(xs)[i] = v[0];
+        for (int t = 0; t < MT; ++t)  // zeros past K
+          v[t] = t < mt && 8 * i < K ? __ldg(reinterpret_cast<const uint4 *>(xm + (int64_t)t * K) + i)
+                                     : make_uint4(0u, 0u, 0u, 0u);
+        if constexpr (MT == 1) {
+          float4 *d = reinterpret_cast<float4 *>(xs) + 2 * i;
+          d[0] = make_float4(half_at(v[0].x, 0), half_at(v[0].x, 1), half_at(v[0].y, 0), half_at(v[0].y, 1));
+          d[1] = make_float4(half_at(v[0].z, 0), half_at(v[0].z, 1), half_at(v[0].w, 0), half_at(v[0].w, 1));
         } else {
 #pragma unroll
           for (int j = 0; j < 8; ++j) {
-            Acts<MT> a;
+            uint32_t *d = reinterpret_cast<uint32_t *>(xs + (8 * i + j) * kES);
 #pragma unroll
-            for (int t = 0; t < MT; ++t) {
-              const uint32_t word = (j >> 1) == 0 ? v[t].x : (j >> 1) == 1 ? v[t].y : (j >> 1) == 2 ? v[t].z : v[t].w;
-              a.h[t] = (unsigned short)(j & 1 ? word >> 16 : word & 0xffffu);
+            for (int t = 0; t < MT; t += 2) {
+              const uint4 &a = v[t], &b = v[t + 1];
+              const uint32_t wa = (j >> 1) == 0 ? a.x : (j >> 1) == 1 ? a.y : (j >> 1) == 2 ? a.z : a.w;
+              const uint32_t wb = (j >> 1) == 0 ? b.x : (j >> 1) == 1 ? b.y : (j >> 1) == 2 ? b.z : b.w;
+              d[t / 2] = __byte_perm(wa, wb, j & 1 ? 0x7632 : 0x5410);
             }
-            xs[8 * i + j] = a;
           }
         }
       }
       __syncthreads();
     }
-    const uint16_t *idx = w.idx;
-    const int nb = (K + kIdxBlock - 1) / kIdxBlock;
-    for (int n = r_lo + warp; n < r_hi; n += kIdxWarps) {
-      const int32_t *offr = w.idx_off + (int64_t)n * nb;
-      int e = __ldg(offr), e1 = __ldg(offr + 1);
-      uint32_t v[kIdxAhead];
+    grid_dep_wait();  // the plane-1 pass (returns at once from the second time on)
+    const int r_lo = b_lo + (b_hi - b_lo) * warp / kIdxWarps, r_hi = b_lo + (b_hi - b_lo) * (warp + 1) / kIdxWarps;
+    if (r_lo >= r_hi) continue;
+    // entries as aligned pairs: entry i is half (i + odd) & 1 of word (i + odd) / 2
+    const int odd = (int)(((uintptr_t)w.idx >> 1) & 1u);
+    const uint32_t *iw = reinterpret_cast<const uint32_t *>(w.idx - odd);
+    const int32_t *offs = w.idx_off + (int64_t)r_lo * nb;
+    const int blocks = (r_hi - r_lo) * nb;
+    auto load_pairs = [&](uint32_t (&v)[kIdxAhead], int e, int e1) {
+      const int first = (e + odd) >> 1, c = ((e1 + odd + 1) >> 1) - first;
+      const uint32_t *q = iw + first + lane;
 #pragma unroll
-      for (int j = 0; j < kIdxAhead; ++j) v[j] = e + lane + 32 * j < e1 ? __ldg(idx + e + lane + 32 * j) : 0u;
+      for (int j = 0; j < kIdxAhead; ++j) v[j] = lane + 32 * j < c && e < e1 ? __ldg(q + 32 * j) : 0u;
+    };
+    // this lane's table entry of row n: codes 27..31 (none in a valid index) weigh nothing
+    const int q = min(lane / 9, 2), d0 = (lane / 3) % 3, d1 = lane % 3;
+    unsigned short h[5];
+    auto load_params = [&](int n) {
+      const unsigned short *mu = reinterpret_cast<const unsigned short *>(w.mu) + (int64_t)n * 4;
+      const unsigned short *a0 = reinterpret_cast<const unsigned short *>(w.a0) + (int64_t)n * 4;
+      h[0] = __ldg(mu + q), h[1] = __ldg(mu + 3), h[2] = __ldg(a0 + q), h[3] = __ldg(a0 + 3);
+      h[4] = q < 2 ? __ldg(reinterpret_cast<const unsigned short *>(w.a1) + (int64_t)n * 2 + q) : (unsigned short)0;
+    };
+    auto h2f = [](unsigned short v) { return __half2float(__ushort_as_half(v)); };
+    load_params(r_lo);
+    int e = __ldg(offs), e1 = __ldg(offs + 1);
+    int e2 = blocks > 1 ? __ldg(offs + 2) : e1;  // the next block's end
+    uint32_t v[kIdxAhead];
+    load_pairs(v, e, e1);
+    int f = 0;  // the block among the run's
+    for (int n = r_lo; n < r_hi; ++n) {
+      float a = (h2f(h[0]) - h2f(h[1])) + (h2f(h[2]) - h2f(h[3])) * (float)(d0 - 1);
+      if (q < 2) a += h2f(h[4]) * (float)(d1 - 1);
       __syncwarp();  // the row before is done with the table
-      {
-        // codes 27..31 (none in a valid index) weigh nothing
-        const int q = lane / 9, d0 = (lane / 3) % 3, d1 = lane % 3;
-        float a = 0.f;
-        if (lane < 27) {
-          const __half *mu = w.mu + (int64_t)n * 4, *a0 = w.a0 + (int64_t)n * 4;
-          a = (__half2float(mu[q]) - __half2float(mu[3])) +
-              (__half2float(a0[q]) - __half2float(a0[3])) * (float)(d0 - 1);
-          if (q < 2) a += __half2float(w.a1[(int64_t)n * 2 + q]) * (float)(d1 - 1);
-        }
-        tab[lane] = a;
-      }
+      tab[lane] = lane < 27 ? a : 0.f;
       __syncwarp();
+      if (n + 1 < r_hi) load_params(n + 1);
+      const int64_t yi = (int64_t)(m0 + lane) * N + n;
+      const float yd = lane < mt && lane < MT ? w.ydense[yi] : 0.f;
       float acc[MT];
 #pragma unroll
       for (int t = 0; t < MT; ++t) acc[t] = 0.f;
-      for (int b = 0; b < nb; ++b) {
-        const int e2 = b + 1 < nb ? __ldg(offr + b + 2) : e1;
+      for (int b = 0; b < nb; ++b, ++f) {
+        const int e3 = f + 2 < blocks ? __ldg(offs + f + 3) : e2;
         uint32_t u[kIdxAhead];  // the next block's entries
-#pragma unroll
-        for (int j = 0; j < kIdxAhead; ++j) u[j] = e1 + lane + 32 * j < e2 ? __ldg(idx + e1 + lane + 32 * j) : 0u;
+        load_pairs(u, e1, e2);
+        const uint32_t xb = xs_a + (uint32_t)b * kBlockBytes;
         const int kb = b * kIdxBlock, kmax = K - 1 - kb;
-        auto add = [&](uint32_t en) {
-          const int k = kb + min((int)(en & (kIdxBlock - 1)), kmax);
-          const float wt = tab[en >> kIdxShift];
-          if (STAGED) {
-            const Acts<MT> a = xs[k];
+        auto add = [&](uint32_t en, bool in) {  // en: the entry in bits 0..15
+          if constexpr (STAGED) {
+            const float wt = lds_f32((en >> 9 & 0x7cu) | tab_a);
+            float x[MT];
+            staged_acts<MT>((en << kESLog & ((kIdxBlock - 1) << kESLog)) | xb, x);
+            if (in) {
 #pragma unroll
-            for (int t = 0; t < MT; ++t) acc[t] = fmaf(wt, __half2float(__ushort_as_half(a.h[t])), acc[t]);
-          } else {
+              for (int t = 0; t < MT; ++t) acc[t] = fmaf(wt, x[t], acc[t]);
+            }
+          } else if (in) {
+            const float wt = tab[en >> kIdxShift & 31u];
+            const int k = kb + min((int)(en & (kIdxBlock - 1)), kmax);
 #pragma unroll
             for (int t = 0; t < MT; ++t)
-              if (t < mt) acc[t] = fmaf(wt, __half2float(__ushort_as_half(__ldg(xm + (int64_t)t * K + k))), acc[t]);
+              if (t < mt) acc[t] = fmaf(wt, h2f(__ldg(xm + (int64_t)t * K + k)), acc[t]);
           }
         };
-        const int c = e1 - e;
+        const int front = (e + odd) & 1, c = e1 - e + front;  // entries from the first word on, the first `front` not ours
 #pragma unroll
         for (int j = 0; j < kIdxAhead; ++j) {
-          if (32 * j >= c) break;
-          if (lane + 32 * j < c) add(v[j]);
+          const int i = 2 * (lane + 32 * j);
+          add(v[j], j == 0 ? i < c && i >= front : i < c);
+          add(v[j] >> 16, i + 1 < c);
         }
-        for (int e0 = e + lane + 32 * kIdxAhead; e0 < e1; e0 += 32) add(__ldg(idx + e0));
-        e = e1;
-        e1 = e2;
+        for (int i = 2 * (lane + 32 * kIdxAhead); i < c; i += 64) {
+          const uint32_t r = __ldg(iw + ((e + odd) >> 1) + (i >> 1));
+          add(r, true);
+          add(r >> 16, i + 1 < c);
+        }
+        e = e1, e1 = e2, e2 = e3;
 #pragma unroll
         for (int j = 0; j < kIdxAhead; ++j) v[j] = u[j];
       }
@@ -424,15 +474,12 @@ __global__ void __launch_bounds__(kIdxThreads, MT == 8 ? 1 : 2)
         for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
         if (lane == t) mine = s;
       }
-      if (!waited) grid_dep_wait();  // the plane-1 pass; what stands above reads only the caller's arrays
-      waited = true;
       if (lane < mt && lane < MT) {
-        const int64_t i = (int64_t)(m0 + lane) * N + n;
-        mine += w.ydense[i];
+        mine += yd;
         if (F32)
-          static_cast<float *>(w.y)[i] = mine;
+          static_cast<float *>(w.y)[yi] = mine;
         else
-          static_cast<__half *>(w.y)[i] = __float2half_rn(mine);
+          static_cast<__half *>(w.y)[yi] = __float2half_rn(mine);
       }
     }
   }
@@ -464,7 +511,7 @@ cudaError_t launch_correct(int M, const Batch<Prob> &bt, int grid, cudaStream_t 
 template <bool F32, int MT, bool STAGED>
 cudaError_t launch_correct_idx(int M, const Batch<Prob> &bt, int64_t total, int rows, int Kmax, int num_sms,
                                cudaStream_t s) {
-  const int smem = kIdxTabBytes + (STAGED ? (int)stage_bytes(Kmax, MT) : 0);
+  const int smem = STAGED ? (int)idx_smem_bytes(Kmax, MT) : kIdxTabBytes;
   const auto kern = correct_idx_kernel<F32, MT, STAGED>;
   const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kIdxMaxSmem);
   if (e != cudaSuccess) return e;
@@ -487,12 +534,12 @@ cudaError_t launch_correct_mt(int M, const Batch<Prob> &bt, int grid, cudaStream
 }
 
 // Tokens per pass: as many as the call has, up to 8, while their staged
-// activations fit a block's shared memory (K up to 14336 for 8 tokens,
-// 114688 for one); beyond that x is gathered from global memory.
+// activations fit a block's shared memory (K up to 12288 for 8 tokens,
+// 55296 for one); beyond that x is gathered from global memory.
 template <bool F32>
 cudaError_t launch_correct_idx_mt(int M, const Batch<Prob> &bt, int64_t total, int rows, int Kmax, int num_sms,
                                   cudaStream_t s) {
-  const auto fits = [&](int MT) { return kIdxTabBytes + stage_bytes(Kmax, MT) <= kIdxMaxSmem; };
+  const auto fits = [&](int MT) { return idx_smem_bytes(Kmax, MT) <= kIdxMaxSmem; };
   if (M > 4 && fits(8)) return launch_correct_idx<F32, 8, true>(M, bt, total, rows, Kmax, num_sms, s);
   if (M > 2 && fits(4)) return launch_correct_idx<F32, 4, true>(M, bt, total, rows, Kmax, num_sms, s);
   if (M > 1 && fits(2)) return launch_correct_idx<F32, 2, true>(M, bt, total, rows, Kmax, num_sms, s);
