@@ -13,6 +13,7 @@
 // per-call views of s1 / off in the workspace (views_kernel), into an fp32
 // buffer.  correct_kernel then adds the second line and writes y.
 #include <algorithm>
+#include <type_traits>
 
 #include "tq_common.cuh"
 #include "tq_launch.cuh"
@@ -47,36 +48,64 @@ struct Prob {
   int32_t N, K, S, blocks;     // blocks = 0: the problem is the other kernel's
   int64_t w_begin;             // N G of the index kernel's problems before it
 };
-template <typename T>
+template <typename T, int CAP = TQ_MAX_BATCH>
 struct Batch {
   int32_t count;
-  T prob[TQ_MAX_BATCH];
+  T prob[CAP];
 };
 static_assert(sizeof(Batch<Prob>) <= 32764 && sizeof(Batch<ViewProb>) <= 32764, "launch parameters");
 
+// fn with the smallest launch parameters that hold bt (31 KB of them cost
+// 1 us more per launch than those of eight problems).
+template <typename T, class Fn>
+cudaError_t with_batch(const Batch<T> &bt, Fn fn) {
+  if (bt.count > kFewProblems) return fn(bt);
+  Batch<T, kFewProblems> few;
+  few.count = bt.count;
+  std::copy(bt.prob, bt.prob + bt.count, few.prob);
+  return fn(few);
+}
+
+constexpr int kViewThreads = 256, kViewUnits = 2;  // views_kernel: 16-byte units of each view per thread
+
 // Block row blockIdx.y = problem: s1 view = alpha0 of mask 3, off view =
-// mu of mask 3 in every group of the row (eight groups per 16-byte store
-// when a row's views are whole 16-byte units); the views' salience words
-// and rowptr are zero (no second plane).
-__global__ void views_kernel(const __grid_constant__ Batch<ViewProb> bt) {
+// mu of mask 3 in every group of the row, eight groups per 16-byte store
+// wherever the rows begin; the views' salience words and rowptr are zero (no
+// second plane).  A small kernel between two launches: it starts while the
+// stream's previous kernel ends, and the prep kernel while it runs.
+template <class BT>
+__global__ void __launch_bounds__(kViewThreads) views_kernel(const __grid_constant__ BT bt) {
+  grid_dep_launch_next();
+  grid_dep_wait();  // the last call's kernels may read these views
   const ViewProb &P = bt.prob[blockIdx.y];
   const int N = P.N, G = P.K / kGroup, W = sal_words_of(P.K);
   const int i0 = blockIdx.x * blockDim.x + threadIdx.x, step = gridDim.x * blockDim.x;
-  const __half *mu = P.mu, *a0 = P.a0;
-  if (G % 8 == 0) {
-    const int G8 = G / 8;
-    uint4 *s1 = reinterpret_cast<uint4 *>(P.s1v), *of = reinterpret_cast<uint4 *>(P.offv);
-    for (int i = i0; i < N * G8; i += step) {
-      const int n = i / G8;
-      const uint32_t a = __half_as_ushort(a0[n * 4 + 3]) * 0x10001u, m = __half_as_ushort(mu[n * 4 + 3]) * 0x10001u;
-      s1[i] = make_uint4(a, a, a, a);
-      of[i] = make_uint4(m, m, m, m);
+  const unsigned short *mu = reinterpret_cast<const unsigned short *>(P.mu);
+  const unsigned short *a0 = reinterpret_cast<const unsigned short *>(P.a0);
+  const int total = N * G, units = (total + 7) / 8;
+  for (int i = i0; i < units; i += step) {
+    int n = 8 * i / G, g = 8 * i - n * G;
+    uint32_t a = __ldg(a0 + (int64_t)n * 4 + 3), m = __ldg(mu + (int64_t)n * 4 + 3);
+    uint32_t av[4], mv[4];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      if (j > 0 && ++g == G) {
+        g = 0;
+        if (++n < N) a = __ldg(a0 + (int64_t)n * 4 + 3), m = __ldg(mu + (int64_t)n * 4 + 3);
+      }
+      av[j / 2] = j & 1 ? av[j / 2] | a << 16 : a;
+      mv[j / 2] = j & 1 ? mv[j / 2] | m << 16 : m;
     }
-  } else {
-    for (int i = i0; i < N * G; i += step) {
-      const int n = i / G;
-      P.s1v[i] = a0[n * 4 + 3];
-      P.offv[i] = mu[n * 4 + 3];
+    if (8 * i + 8 <= total) {
+      reinterpret_cast<uint4 *>(P.s1v)[i] = make_uint4(av[0], av[1], av[2], av[3]);
+      reinterpret_cast<uint4 *>(P.offv)[i] = make_uint4(mv[0], mv[1], mv[2], mv[3]);
+    } else {
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+        if (8 * i + j < total) {
+          P.s1v[8 * i + j] = __ushort_as_half((unsigned short)(av[j / 2] >> (16 * (j & 1))));
+          P.offv[8 * i + j] = __ushort_as_half((unsigned short)(mv[j / 2] >> (16 * (j & 1))));
+        }
     }
   }
   for (int i = i0; i < N * W; i += step) P.salv[i] = 0u;
@@ -329,9 +358,9 @@ __device__ __forceinline__ void staged_acts(uint32_t a, float (&x)[MT]) {
 // step, and 48 us with gathers from global memory.
 // STAGED = false reads x from global memory: K x tokens beyond a block's
 // shared memory.
-template <bool F32, int MT, bool STAGED>
+template <bool F32, int MT, bool STAGED, class BT>
 __global__ void __launch_bounds__(kIdxThreads, MT == 8 ? 1 : 2)
-    correct_idx_kernel(const __grid_constant__ Batch<Prob> bt, int64_t total, int m0, int mt) {
+    correct_idx_kernel(const __grid_constant__ BT bt, int64_t total, int m0, int mt) {
   constexpr int kES = elem_bytes(MT), kBlockBytes = kIdxBlock * kES;
   constexpr int kESLog = MT == 8 ? 4 : MT == 4 ? 3 : 2;
   extern __shared__ __align__(1024) unsigned char smem[];
@@ -512,17 +541,15 @@ template <bool F32, int MT, bool STAGED>
 cudaError_t launch_correct_idx(int M, const Batch<Prob> &bt, int64_t total, int rows, int Kmax, int num_sms,
                                cudaStream_t s) {
   const int smem = STAGED ? (int)idx_smem_bytes(Kmax, MT) : kIdxTabBytes;
-  const auto kern = correct_idx_kernel<F32, MT, STAGED>;
-  const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kIdxMaxSmem);
-  if (e != cudaSuccess) return e;
   const int per_sm = MT < 8 && 2 * (smem + 1024) <= kSmSmem ? 2 : 1;
   const int grid = std::max(1, std::min((rows + kIdxWarps - 1) / kIdxWarps, per_sm * num_sms));
-  for (int m0 = 0; m0 < M; m0 += MT) {
-    const cudaError_t l =
-        launch_dependent_cluster(kern, dim3(grid), 1, kIdxThreads, smem, s, bt, total, m0, std::min(MT, M - m0));
-    if (l != cudaSuccess) return l;
-  }
-  return cudaSuccess;
+  return with_batch(bt, [&](const auto &b) {
+    const auto kern = correct_idx_kernel<F32, MT, STAGED, std::decay_t<decltype(b)>>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kIdxMaxSmem);
+    for (int m0 = 0; m0 < M && e == cudaSuccess; m0 += MT)
+      e = launch_dependent_cluster(kern, dim3(grid), 1, kIdxThreads, smem, s, b, total, m0, std::min(MT, M - m0));
+    return e;
+  });
 }
 
 template <bool F32>
@@ -567,9 +594,11 @@ cudaError_t launch_ew_views(const EwCall *calls, int count, cudaStream_t s) {
     P.K = c.w->K;
     most = std::max<int64_t>(most, (int64_t)P.N * (P.K / kGroup));
   }
-  const int blocks = (int)std::min<int64_t>((most + 255) / 256, 1024);
-  ew::views_kernel<<<dim3(blocks, count), 256, 0, s>>>(bt);
-  return cudaGetLastError();
+  constexpr int64_t per_block = 8 * ew::kViewUnits * ew::kViewThreads;
+  const int blocks = (int)std::min<int64_t>((most + per_block - 1) / per_block, 1024);
+  return ew::with_batch(bt, [&](const auto &b) {
+    return launch_dependent(ew::views_kernel<std::decay_t<decltype(b)>>, dim3(blocks, count), ew::kViewThreads, s, b);
+  });
 }
 
 // Masks 0..2 of every problem added to its plane-1 result, y written: the
