@@ -56,7 +56,7 @@ struct Params {
   int32_t M;            // tokens (rows of every x)
   int32_t total_tiles;  // sum of tiles over problems
   int32_t out_f32;      // y is fp32 (else fp16)
-  int32_t g4_split;     // M <= 2: target groups per work unit of a 256-row tile (0: whole tiles)
+  int32_t g4_split;     // M <= 2: 1: CTAs may share 256-row tiles (y2, tickets zeroed); -1: the sequence kernel
   int32_t general;      // nonzero: the general decode kernels even for M <= 2 (the one-group-per-lane
                         // kernel's operands are then not in the workspace)
   int32_t g4_only;      // nonzero: only the one-group-per-lane kernels read the activation operands

@@ -121,51 +121,61 @@ struct Bars {
 };
 static_assert(sizeof(Bars) <= 256, "barrier block");
 
-// Schedule: CTA c processes global work units [cta_unit[c], cta_unit[c+1]).
-// A unit is one 256-row tile's stages [k nst / u, (k + 1) nst / u), the
-// tile cut into u = min(nst, ceil(G / split)) parts for a target of `split`
-// groups per unit (split = 0: u = 1, whole tiles); units are numbered over
-// the problems in order, tile-major.
+// Schedule: the stages of every tile of every problem, numbered problem by
+// problem and tile by tile, in runs of `run` = ceil(stages / CTAs): CTA c
+// processes the stages [c run, (c + 1) run), beginning with stage local[c] of
+// problem pi[c].  A stage costs the same wherever it is, a tile three to
+// twelve of them: in whole tiles, or tiles cut into parts of at least a CTA's
+// share, one layer of Qwen3-8B left some CTAs with eight stages where 4.8 is
+// even (one token, 10 % salient: 43.7 us, 37.2 in runs; twelve layers 184.8 and
+// 178.6, the 36 of the step 490.3 and 470.4; without a second plane one layer
+// 32.1 and 23.7).  Runs are full but for the last: spread over all CTAs, the
+// 192 stages of a 12288 x 4096 call end no earlier, but four CTAs instead of
+// two add up a tile (18.0 us against 15.0; in parts of a tile 17.1).
 struct Sched {
-  int32_t cta_unit[257];
-  int32_t split;
+  int32_t stages, run;
+  int32_t local[256];
+  uint8_t pi[256];
 };
-__host__ __device__ inline int unit_parts(int K, int SG, int split) {
-  const int G = K / kGroup, nst = nstages(K, SG);
-  return split > 0 ? min(nst, max(1, (G + split - 1) / split)) : 1;
-}
+__host__ __device__ inline int tiles_of(const Problem &P) { return (P.N + kRows - 1) / kRows; }
 
+// A CTA's walk over its stages; what it has of one tile is a segment.
 template <int SG>
 struct Walk {
   const BatchParams *bp;
-  int split, unit, u_end, pi, ub, u, nst, tile, s, s_end;
-  __device__ int parts(int p) const { return unit_parts(bp->prob[p].K, SG, split); }
-  __device__ void locate() {
-    for (;;) {
-      const int U = (bp->prob[pi].N + kRows - 1) / kRows * parts(pi);
-      if (unit < ub + U) break;
-      ub += U;
-      ++pi;
-    }
-    u = parts(pi);
+  int run, k, k_end, pi, nst, tile, s, s_end;
+  bool shared;
+  __device__ void segment() {
+    s_end = min(nst, s + (k_end - k));
+    shared = s > 0 || s_end < nst;
+  }
+  __device__ Walk(const BatchParams *b, const Sched &sc, int cta)
+      : bp(b), run(sc.run), k(cta * sc.run), k_end(min(sc.stages, (cta + 1) * sc.run)), pi(sc.pi[cta]), nst(1), tile(0),
+        s(0), s_end(0), shared(false) {
+    if (k >= k_end) return;
     nst = nstages(bp->prob[pi].K, SG);
-    const int local = unit - ub, k = local % u;
-    tile = local / u;
-    s = k * nst / u;
-    s_end = (k + 1) * nst / u;
+    tile = sc.local[cta] / nst;
+    s = sc.local[cta] - tile * nst;
+    segment();
   }
-  __device__ Walk(const BatchParams *b, int sp, int u0, int u1)
-      : bp(b), split(sp), unit(u0), u_end(u1), pi(0), ub(0), u(1), nst(0), tile(0), s(0), s_end(0) {
-    if (unit < u_end) locate();
-  }
-  __device__ bool valid() const { return unit < u_end; }
+  __device__ bool valid() const { return k < k_end; }
   __device__ const Problem &P() const { return bp->prob[pi]; }
   __device__ int n0() const { return tile * kRows; }
-  __device__ bool last_stage() const { return s + 1 == s_end; }  // of this unit
-  __device__ bool shared_tile() const { return u > 1; }
+  __device__ bool last_stage() const { return s + 1 == s_end; }  // of the segment
+  __device__ bool shared_tile() const { return shared; }
+  // CTAs with stages of the current tile
+  __device__ int owners() const {
+    return (k - s + nst - 1) / run - (k - s) / run + 1;
+  }
   __device__ void next() {
-    if (++s < s_end) return;
-    if (++unit < u_end) locate();
+    ++k;
+    if (++s < s_end || k >= k_end) return;
+    s = 0;
+    if (++tile >= tiles_of(bp->prob[pi])) {
+      tile = 0;
+      nst = nstages(bp->prob[++pi].K, SG);
+    }
+    segment();
   }
 };
 
@@ -456,7 +466,6 @@ __global__ void __launch_bounds__((WD + 1) * 32, 1)
   grid_dep_wait();
   // (the next call's prep kernel is let in only when this one ends: its blocks
   // waiting beside these took the Qwen3-8B step from 492 us to 508)
-  const int t_begin = sc.cta_unit[blockIdx.x], t_end = sc.cta_unit[blockIdx.x + 1];
 
   if (warp < WD) {
     // ============================================================ decode
@@ -479,7 +488,7 @@ __global__ void __launch_bounds__((WD + 1) * 32, 1)
         for (int k = 0; k < MB; ++k) y[t][h][k] = 0.f;
     uint32_t bz[kBSets][4] = {};  // activation registers (zero-column lanes: zero throughout)
     uint32_t buf = 0, phase = 0;
-    for (Walk<SG> w(&bp, sc.split, t_begin, t_end); w.valid(); w.next()) {
+    for (Walk<SG> w(&bp, sc, (int)blockIdx.x); w.valid(); w.next()) {
       const bool ok = __all_sync(0xffffffffu, mm::wait_or_abort(&bars->full[buf], phase, abort_));
       if (!ok) break;
       decode_stage<MB, SG, TL>(dyn, (int)buf, w.s, rA, wb, c, g, realB, tag, bz, y);
@@ -511,7 +520,7 @@ __global__ void __launch_bounds__((WD + 1) * 32, 1)
         } else {
           // a share of the tile's stages: add the partial sums into y2 (fp32
           // atomics, zeroed by the prep kernel); the last of the tile's
-          // units to arrive for this warp's rows writes them
+          // CTAs to arrive for this warp's rows writes them
 #pragma unroll
           for (int t = 0; t < TL; ++t)
 #pragma unroll
@@ -525,7 +534,7 @@ __global__ void __launch_bounds__((WD + 1) * 32, 1)
           __threadfence();
           __syncwarp();
           int last = 0;
-          if (lane == 0) last = atomicAdd(ws_tickets(P, MB) + w.tile * kMaxWarps + warp, 1) == w.u - 1;
+          if (lane == 0) last = atomicAdd(ws_tickets(P, MB) + w.tile * kMaxWarps + warp, 1) == w.owners() - 1;
           if (__shfl_sync(0xffffffffu, last, 0)) {
             __threadfence();
 #pragma unroll
@@ -553,7 +562,7 @@ __global__ void __launch_bounds__((WD + 1) * 32, 1)
     // ========================================================== producer
     uint32_t buf = 0, phase = 0, q = 0;
     int map_pi = -1;
-    for (Walk<SG> w(&bp, sc.split, t_begin, t_end); w.valid(); w.next(), ++q) {
+    for (Walk<SG> w(&bp, sc, (int)blockIdx.x); w.valid(); w.next(), ++q) {
       int ok = 1;
       if (lane == 0) ok = mm::wait_or_abort(&bars->empty[buf], phase ^ 1u, abort_) ? 1 : 0;
       if (!__shfl_sync(0xffffffffu, ok, 0)) break;  // uniform across the warp
@@ -575,6 +584,11 @@ __global__ void __launch_bounds__((WD + 1) * 32, 1)
 __device__ __forceinline__ int share_at(int v, int c, int n) {
   const int q = (int)((unsigned)v / (unsigned)n);
   return q * c + (int)((unsigned)(v - q * n) * (unsigned)c / (unsigned)n);
+}
+// Units of a tile of length K at a target of `split` groups each (0: whole tiles).
+__device__ __forceinline__ int unit_parts(int K, int SG, int split) {
+  const int G = K / kGroup, nst = nstages(K, SG);
+  return split > 0 ? min(nst, max(1, (G + split - 1) / split)) : 1;
 }
 
 // Dependency-ordered sequence of problems (one token): problem p + 1 starts
@@ -1093,51 +1107,27 @@ int64_t g4_workspace_bytes(int M, int N, int K) {
   return g4::pad256(g4::b_bytes(M, K)) + g4::pad256(g4::cs_bytes(M, K)) + g4::pad256(g4::ticket_bytes(N));
 }
 
-// Target groups per work unit for an M <= 2 batch: 0 (whole tiles) when the
-// largest tile costs no more than a CTA's fair share of the batch, else
-// that share, so that no unit holds up the end of the call.
-int g4_split_for(const BatchParams &bp, int num_sms) {
-  const int ctas = std::min(num_sms, 256);
-  int64_t total = 0;
-  int gmax = 0;
-  for (int i = 0; i < bp.count; ++i) {
-    const int G = bp.prob[i].K / kGroup;
-    total += (int64_t)((bp.prob[i].N + g4::kRows - 1) / g4::kRows) * G;
-    gmax = std::max(gmax, G);
-  }
-  const int64_t share = (total + ctas - 1) / ctas;
-  return share >= gmax ? 0 : (int)std::max<int64_t>(1, share);
-}
-
 // The M <= 2 decode kernel over a batch whose prep (activation slots, maps,
 // y2, tickets) and second plane have been launched on the same stream.
 cudaError_t launch_gemv_g4(const BatchParams &bp, int num_sms, cudaStream_t s) {
   thread_local g4::Sched sc;
-  if (!g4::takes(bp) || bp.g4_split < 0) return cudaErrorInvalidValue;
+  if (!g4::takes(bp) || bp.g4_split <= 0) return cudaErrorInvalidValue;
   const int ctas = min(num_sms, 256);
   const int SG = g4::stage_groups(bp.M);
-  sc.split = bp.g4_split;
-  // contiguous unit ranges of about equal cost (groups per unit)
-  int64_t total_cost = 0;
-  for (int i = 0; i < bp.count; ++i) total_cost += (int64_t)((bp.prob[i].N + g4::kRows - 1) / g4::kRows) * (bp.prob[i].K / kGroup);
-  int c = 0, unit = 0;
-  int64_t run2 = 0;  // twice the cost before the current unit
-  sc.cta_unit[0] = 0;
-  for (int i = 0; i < bp.count; ++i) {
-    const int nst = g4::nstages(bp.prob[i].K, SG), G = bp.prob[i].K / kGroup;
-    const int u = g4::unit_parts(bp.prob[i].K, SG, sc.split);
-    const int tiles_i = (bp.prob[i].N + g4::kRows - 1) / g4::kRows;
-    for (int t = 0; t < tiles_i; ++t)
-      for (int k = 0; k < u; ++k, ++unit) {
-        // the unit's groups: its stages' share of G
-        const int64_t s0 = (int64_t)k * nst / u, s1 = (int64_t)(k + 1) * nst / u;
-        const int64_t cost = std::min<int64_t>(G, s1 * SG) - s0 * SG;
-        const int64_t mid2 = run2 + cost;
-        while (c < ctas - 1 && mid2 * ctas >= 2 * total_cost * (int64_t)(c + 1)) sc.cta_unit[++c] = unit;
-        run2 += 2 * cost;
-      }
+  int64_t stages = 0;
+  for (int i = 0; i < bp.count; ++i) stages += (int64_t)g4::tiles_of(bp.prob[i]) * g4::nstages(bp.prob[i].K, SG);
+  if (stages > INT32_MAX / 2) return cudaErrorInvalidValue;
+  sc.stages = (int32_t)stages;
+  sc.run = (int32_t)((stages + ctas - 1) / ctas);
+  int64_t base = 0;  // first stage of problem i
+  for (int i = 0, c = 0; i < bp.count; ++i) {
+    const int64_t next = base + (int64_t)g4::tiles_of(bp.prob[i]) * g4::nstages(bp.prob[i].K, SG);
+    for (; c < ctas && (int64_t)c * sc.run < next; ++c) {
+      sc.pi[c] = (uint8_t)i;
+      sc.local[c] = (int32_t)((int64_t)c * sc.run - base);
+    }
+    base = next;
   }
-  while (c < ctas) sc.cta_unit[++c] = unit;
   using g4::kTL1;
   using g4::kTL2;
   using g4::kWD1;

@@ -200,7 +200,7 @@ __global__ void gemv_mma_prep_kernel(const __grid_constant__ BP params, const __
   // last call's decode kernel, whose workspace this may be) has finished
   // and its writes are visible past this point
   grid_dep_wait();
-  const bool g4_shared = g4::takes(bp) && bp.g4_split > 0;  // split tiles add their partial sums into y2
+  const bool g4_shared = g4::takes(bp) && bp.g4_split > 0;  // shared tiles add their partial sums into y2
   // (the sequence kernel, g4_split < 0, adds every partial sum into y2)
   if (P.nnz > 0 || g4_shared || bp.g4_split < 0) {
     // y2 starts at zero (the indexed second-plane kernel adds into it)
@@ -214,7 +214,7 @@ __global__ void gemv_mma_prep_kernel(const __grid_constant__ BP params, const __
     *reinterpret_cast<int32_t *>(static_cast<unsigned char *>(P.map()) + kSeqCounterOff) = 0;
   }
   if (g4_shared) {
-    // the arrival counters of split tiles start at zero
+    // the arrival counters of shared tiles start at zero
     const int MBx = bp.M;
     int32_t *tk = reinterpret_cast<int32_t *>(P.wsB + P.map_off + kMapSlotBytes + g4::pad256(g4::b_bytes(MBx, P.K)) +
                                               g4::pad256(g4::cs_bytes(MBx, P.K)));
@@ -1350,7 +1350,6 @@ __global__ void __launch_bounds__(kThreads, 1)
 // -------------------------------------------------------------- launcher
 cudaError_t launch_gemv_g4(const BatchParams &bp, int num_sms, cudaStream_t s);
 cudaError_t launch_gemv_p2r(const BatchParams &bp, int num_sms, int32_t *counter, cudaStream_t s);
-int g4_split_for(const BatchParams &bp, int num_sms);
 cudaError_t launch_gemv_seq(const BatchParams &bp, int num_sms, int barrier_extra, bool one, cudaStream_t s);
 
 static int num_sms_mm() {
@@ -1548,10 +1547,10 @@ static bool one_launch(const BatchParams &bp) {
 template <bool F32>
 static cudaError_t launch_mm_one(const BatchParams &bp_in, cudaStream_t s) {
   if (one_launch(bp_in)) return launch_sequence(bp_in, 0, true, s);
-  // the batch with the M <= 2 kernel's tile split filled in
+  // the batch, whose 256-row tiles the M <= 2 kernel's CTAs may share
   thread_local BatchParams bp;
   copy_params(bp, bp_in);
-  bp.g4_split = g4::takes(bp) ? g4_split_for(bp, num_sms_mm()) : 1;
+  bp.g4_split = 1;
   thread_local mm::Sched sc;
   if (bp.M < 1 || bp.M > 16 || mm::Layout(bp.M).used2 > mm::kArena2) return cudaErrorInvalidValue;
   const int ctas = min(num_sms_mm(), 256);

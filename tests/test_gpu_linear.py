@@ -334,3 +334,28 @@ def test_batched_parameter_sizes(H, count, M, index):
     H.device_status_ok()
     for (_, _, y), (y_ref, a_ref) in zip(items, refs):
         H.assert_close(y.float().cpu().numpy().astype(np.float64), y_ref, a_ref)
+
+
+@pytest.mark.parametrize("M", [1, 2])
+@pytest.mark.parametrize("frac", [0.0, 0.1])
+@pytest.mark.parametrize("shapes", [
+    [(3000, 4224), (130, 12288), (513, 640), (1, 128), (4096, 1024)],  # runs that begin and end inside tiles
+    [(600, 12288)],                                                    # fewer stages than CTAs
+    [(2560, 4096)] * 12,                                               # runs that cover whole tiles between shared ones
+])
+def test_batched_shared_tiles(H, M, frac, shapes):
+    from paper_2609_09240_gb300 import tq
+    items, refs = [], []
+    for i, (N, K) in enumerate(shapes):
+        w = wl.gen_weights(N, K, frac, config=6, proj=40 + i)
+        x = wl.gen_x(M, K, config=6, proj=40 + i)
+        refs.append(H.oracle_ref(w, x))
+        items.append((H.pack_on_gpu(w, index=i % 4 != 3), H.dev(x),
+                      torch.empty((M, N), dtype=torch.float16, device="cuda")))
+    for _ in range(2):
+        for _, _, y in items:
+            y.fill_(float("nan"))
+        tq.tq_linear_batched(tq.Batch(M, items))
+        H.device_status_ok()
+        for (_, _, y), (y_ref, a_ref) in zip(items, refs):
+            H.assert_close(y.float().cpu().numpy().astype(np.float64), y_ref, a_ref)
