@@ -22,6 +22,7 @@
 #include <cudaTypedefs.h>
 
 #include "tq_common.cuh"
+#include "tq_launch.cuh"
 #include "tq_sm100.cuh"
 
 namespace tq {
@@ -155,6 +156,14 @@ __device__ __forceinline__ int cm_off(int row, int e) { return ((row >> 3) * 16 
 //  * warp 17 (one thread): per stage 4 TT MMAs (M = 128 rows, N = 256
 //    tokens, K = 16; token half t into tensor-memory columns 256 t ..);
 //  * at the end warps 0..15 read the accumulators and write y.
+// SPLIT: the CTAs of a cluster share a tile, each over its share of the
+// groups.  They then exchange partial sums through distributed shared memory
+// (each takes an equal share of the token columns, the others write theirs
+// into its rings, which are free by then), add them in rank order and write y.
+// A few-token call has a CTA per 128 rows, each held up by its decoders; on an
+// otherwise idle chip the share of the groups is the time: 64 tokens x 1024 x
+// 4096 15.9 us with eight CTAs per tile (49.8 with one), 256 x 4096 x 4096
+// 23.6 with four (51.2), 200 x 9728 x 2560 26.9 with two (34.8).
 // A decoded weight tile serves 256 TT tokens and 8 TT MMAs: with TT = 2
 // every weight is decoded once per 512 tokens.  Needs a tensor map of x
 // that the host encodes (x 16-byte aligned, K a multiple of 128).
@@ -203,20 +212,37 @@ struct Bars2 {
 };
 static_assert(sizeof(Bars2) <= 256, "prefill2 barriers");
 
-template <bool F32, int TT>
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// a float into another cluster CTA's shared memory, at this CTA's address a
+__device__ __forceinline__ void st_remote(uint32_t a, int rank, float v) {
+  asm volatile("{\n.reg .b32 r;\nmapa.shared::cluster.u32 r, %0, %1;\nst.shared::cluster.f32 [r], %2;\n}" ::"r"(a),
+               "r"(rank), "f"(v)
+               : "memory");
+}
+constexpr int kMaxSplit = 8;  // CTAs of a cluster
+static_assert((kMaxSplit - 1) * (BT2 / kMaxSplit) * BR2 * 4 <= Lay2<1>::oP, "the exchanged sums fit the rings");
+
+template <bool F32, int TT, bool SPLIT>
 __global__ void __launch_bounds__(kThreads2, 1)
-    prefill2_kernel(const __grid_constant__ PfBatch B, int M) {
+    prefill2_kernel(const __grid_constant__ PfBatch B, int M, int split) {
   using L = Lay2<TT>;
   extern __shared__ __align__(1024) unsigned char smem[];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  // this CTA's problem and tile
+  static_assert(!SPLIT || TT == 1, "shared tiles are 256 tokens wide");
+  // this CTA's problem and tile (and its rank among those sharing it)
+  const int tile = SPLIT ? (int)blockIdx.x / split : (int)blockIdx.x;
+  const int rank = SPLIT ? (int)blockIdx.x - tile * split : 0;
   int pi = 0;
-  while (pi + 1 < B.count && B.tile_begin[pi + 1] <= (int)blockIdx.x) ++pi;
+  while (pi + 1 < B.count && B.tile_begin[pi + 1] <= tile) ++pi;
   const Problem &P = B.prob[pi];
   const CUtensorMap *xmap = &B.xmap[pi], *pmap = &B.pmap[pi];
-  const int local = (int)blockIdx.x - B.tile_begin[pi];
+  const int local = tile - B.tile_begin[pi];
   const int m0 = (local % B.mtiles) * (TT * BT2), n0 = (local / B.mtiles) * BR2;
-  const int N = P.N, G = P.K / kGroup;
+  const int N = P.N, Gall = P.K / kGroup;
+  const int gb = SPLIT ? Gall * rank / split : 0;                  // the CTA's first group
+  const int G = SPLIT ? Gall * (rank + 1) / split - gb : Gall;     // and how many it has
   uint64_t *sel = reinterpret_cast<uint64_t *>(smem + L::oSel);
   Bars2 *bars = reinterpret_cast<Bars2 *>(smem + L::oBar);
   volatile int32_t *abort_ = &bars->abort_;
@@ -243,6 +269,7 @@ __global__ void __launch_bounds__(kThreads2, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = bars->tmem_slot;
+  if (SPLIT) grid_dep_wait();  // launched programmatically
 
   if (warp < kDecWarps2) {
     // ======================================================= weight decode
@@ -258,16 +285,22 @@ __global__ void __launch_bounds__(kThreads2, 1)
     const uint32_t *salrow = P.sal + (int64_t)(valid ? n : 0) * W;
     int64_t j = (valid && P.nnz > 0) ? P.rowptr[n] : 0;
     uint32_t salw = (valid && P.nnz > 0) ? __ldg(salrow) : 0u;
-    const bool vec8 = (G % 8) == 0 && ((((uintptr_t)P.s1) | ((uintptr_t)P.off)) & 15u) == 0;
-    const unsigned short *s1h = reinterpret_cast<const unsigned short *>(P.s1) + (int64_t)(valid ? n : 0) * G;
-    const unsigned short *ofh = reinterpret_cast<const unsigned short *>(P.off) + (int64_t)(valid ? n : 0) * G;
+    if (SPLIT && valid && P.nnz > 0) {
+      // the records of the row's groups before gb
+      for (int i = 0; i < gb >> 5; ++i) j += __popc(__ldg(salrow + i));
+      salw = __ldg(salrow + (gb >> 5));
+      j += __popc(salw & ((1u << (gb & 31)) - 1u));
+    }
+    const bool vec8 = (Gall % 8) == 0 && ((((uintptr_t)P.s1) | ((uintptr_t)P.off)) & 15u) == 0;
+    const unsigned short *s1h = reinterpret_cast<const unsigned short *>(P.s1) + (int64_t)(valid ? n : 0) * Gall;
+    const unsigned short *ofh = reinterpret_cast<const unsigned short *>(P.off) + (int64_t)(valid ? n : 0) * Gall;
     uint4 s1v = make_uint4(0u, 0u, 0u, 0u), ofv = make_uint4(0u, 0u, 0u, 0u);
     // everything of group g but its plane-1 bytes
     auto fetch = [&](int g, RowGroup &nx) {
       if (vec8) {
-        if ((g & 7) == 0 && valid) {
-          s1v = __ldg(reinterpret_cast<const uint4 *>(s1h + g));
-          ofv = __ldg(reinterpret_cast<const uint4 *>(ofh + g));
+        if (((g & 7) == 0 || (SPLIT && g == gb)) && valid) {
+          s1v = __ldg(reinterpret_cast<const uint4 *>(s1h + (SPLIT ? g & ~7 : g)));
+          ofv = __ldg(reinterpret_cast<const uint4 *>(ofh + (SPLIT ? g & ~7 : g)));
         }
         const int k = g & 7;
         const uint32_t ws1 = k < 2 ? s1v.x : k < 4 ? s1v.y : k < 6 ? s1v.z : s1v.w;
@@ -278,7 +311,7 @@ __global__ void __launch_bounds__(kThreads2, 1)
         nx.s1 = valid ? __ldg(s1h + g) : (unsigned short)0;
         nx.of = valid ? __ldg(ofh + g) : (unsigned short)0;
       }
-      if ((g & 31) == 0 && g > 0 && valid && P.nnz > 0) salw = __ldg(salrow + (g >> 5));
+      if ((g & 31) == 0 && g > gb && valid && P.nnz > 0) salw = __ldg(salrow + (g >> 5));
       nx.salient = (salw >> (g & 31)) & 1u;
       nx.s2 = 0;
       nx.rodd = false;
@@ -297,8 +330,8 @@ __global__ void __launch_bounds__(kThreads2, 1)
       }
     };
     RowGroup nx;
-    fetch(0, nx);
-    for (int g = 0; g < G; ++g) {
+    fetch(gb, nx);
+    for (int g = 0; g < G; ++g) {  // group gb + g
       const int s = g % NW2, ps = g % NP2;
       if (g >= NW2 && !__all_sync(0xffffffffu, wait_or_abort(&bars->wempty[s], ((uint32_t)(g / NW2) & 1u) ^ 1u, abort_)))
         break;
@@ -309,15 +342,15 @@ __global__ void __launch_bounds__(kThreads2, 1)
         const uint4 *pw = reinterpret_cast<const uint4 *>(smem + L::oP + ps * kPSlot2 + r * kPRow2);
         const uint4 a0 = pw[0], a1 = pw[1], a2 = pw[2];
         const uint32_t w[12] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w, a2.x, a2.y, a2.z, a2.w};
-        const int q = ((kGroupBytes * g) & 15) >> 2;
+        const int q = ((kGroupBytes * (gb + g)) & 15) >> 2;
         uint32_t t[10];
 #pragma unroll
         for (int i = 0; i < 10; ++i) t[i] = (q & 2) ? w[i + 2] : w[i];
 #pragma unroll
         for (int i = 0; i < 7; ++i) cur.r8[i] = (q & 1) ? t[i + 1] : t[i];
-        cur.odd = g & 1;  // the group starts 2 bytes into its first word
+        cur.odd = (gb + g) & 1;  // the group starts 2 bytes into its first word
       }
-      if (g + 1 < G) fetch(g + 1, nx);
+      if (g + 1 < G) fetch(gb + g + 1, nx);
       uint32_t wv[16];
       if (qq == 0)
         decode_row_quarter<0>(cur, sel, wv);
@@ -352,7 +385,7 @@ __global__ void __launch_bounds__(kThreads2, 1)
         asm volatile(
             "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(
                 smem_u32(smem + L::oP + sl * kPSlot2)),
-            "l"(pmap), "r"((kGroupBytes * g) & ~15), "r"(n0), "r"(smem_u32(&bars->pfull[sl]))
+            "l"(pmap), "r"((kGroupBytes * (gb + g)) & ~15), "r"(n0), "r"(smem_u32(&bars->pfull[sl]))
             : "memory");
         ++issued;
       }
@@ -371,7 +404,7 @@ __global__ void __launch_bounds__(kThreads2, 1)
           asm volatile(
               "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(
                   smem_u32(smem + L::oX + sl * L::kXStage + t * kXHalf2)),
-              "l"(xmap), "r"(xs * XK2), "r"(m0 + t * BT2), "r"(smem_u32(&bars->xfull[sl]))
+              "l"(xmap), "r"(gb * BK + xs * XK2), "r"(m0 + t * BT2), "r"(smem_u32(&bars->xfull[sl]))
               : "memory");
         ++issued;
       }
@@ -416,31 +449,69 @@ __global__ void __launch_bounds__(kThreads2, 1)
 
   // ================================================================ epilogue
   __syncwarp();
+  bool ok = false;
   if (warp < kDecWarps2) {
-    const bool ok = __all_sync(0xffffffffu, wait_or_abort(&bars->done, 0u, abort_));
+    ok = __all_sync(0xffffffffu, wait_or_abort(&bars->done, 0u, abort_));
     tc_fence_after();
-    if (ok) {
-      // 16 warps: tensor-memory lane quarter q (rows 32 q ..), then a
-      // quarter of the 256 TT token columns
-      const int q = warp & 3, part = warp >> 2;  // 0..3
-      const int cb = part * (TT * BT2 / 4), ce = cb + TT * BT2 / 4;
-      const int n = n0 + 32 * q + lane;
-#pragma unroll 1
-      for (int c0 = cb; c0 < ce; c0 += 8) {
-        uint32_t v[8];
-        tmem_ld8(tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)c0, v);
-        tmem_wait_ld();
-        if (n < N) {
+  }
+  // 16 warps: tensor-memory lane quarter q (rows 32 q ..), then a quarter of
+  // the 256 TT token columns (SPLIT: of the columns of each CTA)
+  const int q = warp & 3, part = warp >> 2;
+  const int n = n0 + 32 * q + lane;
+  auto store = [&](int m, float v) {
+    if (F32)
+      static_cast<float *>(P.y)[(int64_t)m * N + n] = v;
+    else
+      static_cast<__half *>(P.y)[(int64_t)m * N + n] = __float2half_rn(v);
+  };
+  if constexpr (SPLIT) {
+    const int cols = BT2 / split, cw = cols / 4;  // columns of a CTA, of a warp
+    const uint32_t ex = smem_u32(smem) + (uint32_t)(32 * q + lane) * 4u;  // sums [from][column][row]
+    auto slot = [&](int from, int to, int c) -> uint32_t {
+      return (uint32_t)(((from < to ? from : from - 1) * cols + c) * BR2 * 4);
+    };
+    cluster_sync();  // every CTA is done with its rings
+    if (warp < kDecWarps2 && ok) {
+      for (int d = 1; d < split; ++d) {
+        const int to = (rank + d) % split;
+        for (int c = part * cw; c < (part + 1) * cw && m0 + to * cols + c < M; c += 8) {
+          uint32_t v[8];
+          tmem_ld8(tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(to * cols + c), v);
+          tmem_wait_ld();
 #pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            const int m = m0 + c0 + i;
-            if (m < M) {
-              if (F32)
-                static_cast<float *>(P.y)[(int64_t)m * N + n] = __uint_as_float(v[i]);
-              else
-                static_cast<__half *>(P.y)[(int64_t)m * N + n] = __float2half_rn(__uint_as_float(v[i]));
-            }
-          }
+          for (int i = 0; i < 8; ++i) st_remote(ex + slot(rank, to, c + i), to, __uint_as_float(v[i]));
+        }
+      }
+    }
+    cluster_sync();  // the sums have arrived
+    if (warp < kDecWarps2 && ok) {
+      for (int c = part * cw; c < (part + 1) * cw && m0 + rank * cols + c < M; c += 8) {
+        uint32_t v[8];
+        tmem_ld8(tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(rank * cols + c), v);
+        tmem_wait_ld();
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          float sum = 0.f;
+          for (int from = 0; from < split; ++from)
+            sum += from == rank ? __uint_as_float(v[i])
+                                : *reinterpret_cast<const float *>(smem + slot(from, rank, c + i) + (32 * q + lane) * 4);
+          const int m = m0 + rank * cols + c + i;
+          if (n < N && m < M) store(m, sum);
+        }
+      }
+    }
+  } else if (warp < kDecWarps2 && ok) {
+    const int cb = part * (TT * BT2 / 4), ce = cb + TT * BT2 / 4;
+#pragma unroll 1
+    for (int c0 = cb; c0 < ce; c0 += 8) {
+      uint32_t v[8];
+      tmem_ld8(tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)c0, v);
+      tmem_wait_ld();
+      if (n < N) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const int m = m0 + c0 + i;
+          if (m < M) store(m, __uint_as_float(v[i]));
         }
       }
     }
@@ -499,6 +570,34 @@ static bool encode_p_map(const void *plane1, int N, int K, int rows, CUtensorMap
                 CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// Clusters of 2, 4 or 8 CTAs of the split kernel that the chip runs at once
+// (0 where that cannot be told: no split).
+static int max_clusters(int split) {
+  struct Counts {
+    int n[pf::kMaxSplit + 1] = {};
+    Counts() {
+      const auto kern = pf::prefill2_kernel<false, 1, true>;
+      if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, pf::Lay2<1>::kSmem) != cudaSuccess)
+        return;
+      for (int c = 2; c <= pf::kMaxSplit; c *= 2) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(c);
+        cfg.blockDim = dim3(pf::kThreads2);
+        cfg.dynamicSmemBytes = pf::Lay2<1>::kSmem;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = c;
+        attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        if (cudaOccupancyMaxActiveClusters(&n[c], kern, &cfg) != cudaSuccess) n[c] = 0;
+      }
+    }
+  };
+  static const Counts counts;
+  return counts.n[split];
+}
+
 // One launch over `count` (<= kPfMaxBatch) problems sharing M: 512-token
 // tiles (each weight decoded once per 512 tokens) unless the tokens fit one
 // 256-token tile or twice as many 256-token CTAs still fit in one wave.
@@ -525,12 +624,27 @@ static cudaError_t launch_prefill_group(const Problem *probs, int count, int M, 
     B.prob[k] = P;
     B.tile_begin[k + 1] = B.tile_begin[k] + (P.N + pf::BR2 - 1) / pf::BR2 * B.mtiles;
   }
-  auto kern = wide ? (f32 ? pf::prefill2_kernel<true, 2> : pf::prefill2_kernel<false, 2>)
-                   : (f32 ? pf::prefill2_kernel<true, 1> : pf::prefill2_kernel<false, 1>);
+  // CTAs per tile: the most whose clusters all run at once (more would wait
+  // for the first to end: 16 clusters of eight for 512 tokens x 1024 x 2560
+  // took 29.2 us, of four 18.5), two groups each at least
+  int split = 1;
+  int gmin = probs[0].K / kGroup;
+  for (int i = 1; i < count; ++i) gmin = std::min(gmin, probs[i].K / kGroup);
+  const int64_t tiles = B.tile_begin[count];
+  while (!wide && 2 * split <= pf::kMaxSplit && gmin >= 4 * split && tiles <= max_clusters(2 * split)) split *= 2;
+  if (split > 1) {
+    auto kern = f32 ? pf::prefill2_kernel<true, 1, true> : pf::prefill2_kernel<false, 1, true>;
+    const int smem = pf::Lay2<1>::kSmem;
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
+    return launch_dependent_cluster(kern, dim3((unsigned)tiles * split), split, pf::kThreads2, smem, s, B, M, split);
+  }
+  auto kern = wide ? (f32 ? pf::prefill2_kernel<true, 2, false> : pf::prefill2_kernel<false, 2, false>)
+                   : (f32 ? pf::prefill2_kernel<true, 1, false> : pf::prefill2_kernel<false, 1, false>);
   const int smem = wide ? pf::Lay2<2>::kSmem : pf::Lay2<1>::kSmem;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
-  kern<<<B.tile_begin[count], pf::kThreads2, smem, s>>>(B, M);
+  kern<<<B.tile_begin[count], pf::kThreads2, smem, s>>>(B, M, 1);
   return cudaGetLastError();
 }
 

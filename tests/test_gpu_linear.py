@@ -359,3 +359,32 @@ def test_batched_shared_tiles(H, M, frac, shapes):
         H.device_status_ok()
         for (_, _, y), (y_ref, a_ref) in zip(items, refs):
             H.assert_close(y.float().cpu().numpy().astype(np.float64), y_ref, a_ref)
+
+
+@pytest.mark.parametrize("M,shapes", [
+    (17, [(128, 1024)]),                                # four CTAs of two groups; one with real tokens
+    (200, [(1000, 4224)]),                              # eight CTAs, 33 groups: shares that begin anywhere in a salience word
+    (300, [(1000, 1152)]),                              # two token tiles
+    (256, [(9728, 640)]),                               # two CTAs for every SM of the chip
+    (129, [(129, 12288)]),
+    (33, [(300, 2560), (1, 1024), (257, 4096)]),        # a batch of different lengths
+    (40, [(300, 384)]),                                 # too few groups to share
+])
+@pytest.mark.parametrize("frac,f32", [(0.3, False), (0.0, True)])
+def test_prefill_shared_tiles(H, M, shapes, frac, f32):
+    from paper_2609_09240_gb300 import tq
+    items, refs = [], []
+    for i, (N, K) in enumerate(shapes):
+        w = wl.gen_weights(N, K, frac, config=6, proj=60 + i)
+        x = wl.gen_x(M, K, config=6, proj=60 + i)
+        refs.append(H.oracle_ref(w, x))
+        items.append((H.pack_on_gpu(w), H.dev(x), torch.empty((M, N), dtype=torch.float16, device="cuda")))
+    if len(items) > 1:
+        tq.tq_linear_batched(tq.Batch(M, items))
+        ys = [y for _, _, y in items]
+    else:
+        pw, x, _ = items[0]
+        ys = [(tq.tq_linear_f32out if f32 else tq.tq_linear)(x, pw)]
+    H.device_status_ok()
+    for y, (y_ref, a_ref) in zip(ys, refs):
+        H.assert_close(y.float().cpu().numpy().astype(np.float64), y_ref, a_ref)
