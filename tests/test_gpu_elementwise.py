@@ -282,3 +282,23 @@ def test_linear_indexed_runs_and_staging(H, M, N, K, cover):
     y = tq.tq_ew_linear(H.dev(xb), _indexed(H, w))
     H.device_status_ok()
     H.assert_close(y.float().cpu().numpy()[:, rows].astype(np.float64), y_ref, a_ref)
+
+
+@pytest.mark.parametrize("M,N,K", [(1, 37, 2176), (4, 300, 4096)])
+def test_linear_indexed_odd_index_address(H, M, N, K):
+    """Index entries need two-byte alignment only: the kernel's pairs then begin
+    one entry before the array."""
+    from paper_2609_09240_gb300 import tq
+    w = wl.gen_ew_weights(N, K, config=26, proj=M)
+    x = H.dev(wl.gen_x(M, K, config=26, proj=M))
+    g = _indexed(H, w)
+    y = tq.tq_ew_linear(x, g)
+    moved = torch.zeros(g.idx.numel() + 1, dtype=g.idx.dtype, device="cuda")
+    moved[1:] = g.idx
+    g.idx = moved[1:]
+    assert g.idx.data_ptr() % 4 == 2
+    mp, p1, rp, p2, st = ew.pack(w.T0, w.T1, w.mask)
+    y_ref, a_ref = ew.linear(wl.gen_x(M, K, config=26, proj=M), K, mp, p1, rp, p2, w.mu, w.a0, w.a1)
+    for out in (y, tq.tq_ew_linear(x, g)):
+        H.device_status_ok()
+        H.assert_close(out.float().cpu().numpy().astype(np.float64), y_ref, a_ref)
