@@ -1512,6 +1512,7 @@ static cudaError_t launch_mm(const BatchParams &bp, cudaStream_t s) {
     sub.count = j - i;
     sub.M = bp.M;
     sub.out_f32 = bp.out_f32;
+    sub.general = bp.general;  // the workspace's layout is the batch's
     int tiles = 0;
     for (int k = 0; k < sub.count; ++k) {
       sub.prob[k] = bp.prob[i + k];

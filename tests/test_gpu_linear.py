@@ -134,6 +134,27 @@ def test_batched_many_row_lengths(H):
         H.assert_close(y.float().cpu().numpy(), y_ref, a_ref)
 
 
+@pytest.mark.parametrize("index", ["all", "none", "some"])
+@pytest.mark.parametrize("M", [1, 2, 9, 10, 12])
+def test_batched_many_row_lengths_tokens(H, M, index):
+    """Twelve templates in six problems, so that the batch runs as sub-batches;
+    without every index, nine and ten tokens leave one and two for a second
+    pass in the general layout."""
+    from paper_2609_09240_gb300 import tq
+    items, refs = [], []
+    for i in range(6):
+        N, K = 100 + 60 * i, 1024 * (1 + i % 3)
+        w = wl.gen_weights(N, K, 0.2, config=6, proj=80 + i)
+        x = wl.gen_x(M, K, config=6, proj=80 + i)
+        refs.append(H.oracle_ref(w, x))
+        items.append((H.pack_on_gpu(w, index=index == "all" or (index == "some" and i % 2 == 1)), H.dev(x),
+                      torch.full((M, N), float("nan"), dtype=torch.float16, device="cuda")))
+    tq.tq_linear_batched(tq.Batch(M, items))
+    H.device_status_ok()
+    for (_, _, y), (y_ref, a_ref) in zip(items, refs):
+        H.assert_close(y.float().cpu().numpy(), y_ref, a_ref)
+
+
 @pytest.mark.parametrize("index", [True, False])
 @pytest.mark.parametrize("M", [1, 3])
 def test_batched_max_problems(H, M, index):
