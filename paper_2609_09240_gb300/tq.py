@@ -185,8 +185,12 @@ def _p(t):
 def _stream(stream):
     if stream is None:
         # the current stream's handle without a Stream object around it (0.4 us
-        # a call instead of 3.0; every caller's tensors have initialized CUDA)
-        return ctypes.c_void_p(torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice()))
+        # a call instead of 3.0; every caller's tensors have initialized CUDA);
+        # a torch without these private functions gives the object
+        try:
+            return ctypes.c_void_p(torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice()))
+        except AttributeError:
+            stream = torch.cuda.current_stream()
     return ctypes.c_void_p(stream.cuda_stream)
 
 

@@ -142,3 +142,19 @@ def test_binding_argument_counts_match_the_header():
         assert len(fn.argtypes) == n, (name, len(fn.argtypes), n)
         checked += 1
     assert checked >= 25
+
+
+def test_current_stream_without_private_names(monkeypatch):
+    """A torch without the raw-stream functions: the public stream object."""
+    import types
+
+    import torch
+    from paper_2609_09240_gb300 import tq
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: types.SimpleNamespace(cuda_stream=0x1230))
+    for name in ("_cuda_getCurrentRawStream", "_cuda_getDevice"):
+        with monkeypatch.context() as m:
+            m.setattr(torch._C, "_cuda_getCurrentRawStream", lambda d: 0x4560, raising=False)
+            m.setattr(torch._C, "_cuda_getDevice", lambda: 0, raising=False)
+            assert tq._stream(None).value == 0x4560
+            m.delattr(torch._C, name)
+            assert tq._stream(None).value == 0x1230
