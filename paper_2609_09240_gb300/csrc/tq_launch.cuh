@@ -1,5 +1,7 @@
 // Kernel launches.
 #pragma once
+#include <atomic>
+
 #include <cuda_runtime.h>
 
 namespace tq {
@@ -38,6 +40,40 @@ inline cudaError_t launch_big_smem(void (*kern)(P...), int ctas, int threads, in
   const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
   return launch_dependent_cluster(kern, dim3(ctas), 1, threads, smem, s, args...);
+}
+
+// Clusters of `cluster` (up to 16) CTAs of KERN, each with `smem` bytes of
+// dynamic shared memory, that the current device runs at once; 0 where it
+// holds none or that cannot be told (a partition whose GPCs have fewer SMs, a
+// failing query: its error does not stay behind for the caller's next check).
+// A kernel asks for one smem only; devices are asked once.
+template <auto KERN>
+int clusters_at_once(int cluster, int threads, int smem) {
+  constexpr int kDevices = 64;
+  static std::atomic<int> known[kDevices][17];  // clusters + 1, 0: not asked yet
+  int dev = -1;
+  if (cudaGetDevice(&dev) != cudaSuccess) dev = -1;
+  std::atomic<int> *slot = dev >= 0 && dev < kDevices ? &known[dev][cluster] : nullptr;
+  if (slot && slot->load(std::memory_order_relaxed)) return slot->load(std::memory_order_relaxed) - 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(cluster);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = cluster;
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  int n = 0;
+  if (dev < 0 || cudaFuncSetAttribute(KERN, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
+      (cluster > 8 && cudaFuncSetAttribute(KERN, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) ||
+      cudaOccupancyMaxActiveClusters(&n, KERN, &cfg) != cudaSuccess) {
+    (void)cudaGetLastError();
+    n = 0;
+  }
+  if (slot) slot->store(n + 1, std::memory_order_relaxed);
+  return n;
 }
 
 }  // namespace tq

@@ -570,34 +570,6 @@ static bool encode_p_map(const void *plane1, int N, int K, int rows, CUtensorMap
                 CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// Clusters of 2, 4 or 8 CTAs of the split kernel that the chip runs at once
-// (0 where that cannot be told: no split).
-static int max_clusters(int split) {
-  struct Counts {
-    int n[pf::kMaxSplit + 1] = {};
-    Counts() {
-      const auto kern = pf::prefill2_kernel<false, 1, true>;
-      if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, pf::Lay2<1>::kSmem) != cudaSuccess)
-        return;
-      for (int c = 2; c <= pf::kMaxSplit; c *= 2) {
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(c);
-        cfg.blockDim = dim3(pf::kThreads2);
-        cfg.dynamicSmemBytes = pf::Lay2<1>::kSmem;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = c;
-        attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        if (cudaOccupancyMaxActiveClusters(&n[c], kern, &cfg) != cudaSuccess) n[c] = 0;
-      }
-    }
-  };
-  static const Counts counts;
-  return counts.n[split];
-}
-
 // One launch over `count` (<= kPfMaxBatch) problems sharing M: 512-token
 // tiles (each weight decoded once per 512 tokens) unless the tokens fit one
 // 256-token tile or twice as many 256-token CTAs still fit in one wave.
@@ -631,7 +603,10 @@ static cudaError_t launch_prefill_group(const Problem *probs, int count, int M, 
   int gmin = probs[0].K / kGroup;
   for (int i = 1; i < count; ++i) gmin = std::min(gmin, probs[i].K / kGroup);
   const int64_t tiles = B.tile_begin[count];
-  while (!wide && 2 * split <= pf::kMaxSplit && gmin >= 4 * split && tiles <= max_clusters(2 * split)) split *= 2;
+  const auto at_once = [](int c) {
+    return clusters_at_once<pf::prefill2_kernel<false, 1, true>>(c, pf::kThreads2, pf::Lay2<1>::kSmem);
+  };
+  while (!wide && 2 * split <= pf::kMaxSplit && gmin >= 4 * split && tiles <= at_once(2 * split)) split *= 2;
   if (split > 1) {
     auto kern = f32 ? pf::prefill2_kernel<true, 1, true> : pf::prefill2_kernel<false, 1, true>;
     const int smem = pf::Lay2<1>::kSmem;
