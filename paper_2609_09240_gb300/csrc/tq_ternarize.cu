@@ -27,9 +27,10 @@
 //                       largest key, the salience words (keys above the
 //                       selected key, and the first `need` equal keys in
 //                       block-id order) and rowptr, in one cluster; if the
-//                       keys exceed its shared memory instead, over the whole
-//                       chip, tern_hist_kernel (a pass each; the last CTA to
-//                       finish picks the digit, no CTA waits for another),
+//                       keys exceed its shared memory or the device holds no
+//                       such cluster, instead, over the whole chip,
+//                       tern_hist_kernel (a pass each; the last CTA to finish
+//                       picks the digit, no CTA waits for another),
 //                       tern_count_kernel (keys equal to the selected one, per
 //                       chunk of salience words), tern_mark_kernel and rowptr
 //                       (tq_codec.cu); then
@@ -395,7 +396,8 @@ __global__ void __launch_bounds__(kMarkThreads) tern_mark_kernel(int NW, int G, 
 // with programmatic dependent launches), this 30.  Taken while the keys fit
 // (about 850,000 blocks if the groups are a multiple of 32); with eight CTAs
 // it took 43 us, and digits of 11 bits (three barriers, but 2048 bins to add
-// up over 16 CTAs) 48.
+// up over 16 CTAs) 48.  A cluster of 16 is not a portable size: a device (a
+// partition of one) whose GPCs have fewer SMs takes the separate kernels.
 constexpr int kSelCtas = 16, kSelWarps = kSelThreads / 32, kSelBatch = 8;
 constexpr int kSelCopies = 8;    // of the first digit's histogram (all keys, in a few bins),
 constexpr int kSelStride = 257;  // on different banks
@@ -730,7 +732,10 @@ cudaError_t launch_ternarize(int N, int K, const uint16_t *W, int64_t nnz, int s
   uint32_t *keys = reinterpret_cast<uint32_t *>(ws + pad(NB * 16));
   SelWork *sw = reinterpret_cast<SelWork *>(ws + pad(NB * 16) + pad(NB * 4));
   uint32_t *chunk_eq = reinterpret_cast<uint32_t *>(ws + pad(NB * 16) + pad(NB * 4) + pad(sizeof(SelWork)));
-  const bool cluster = nnz > 0 && select_keys(N, SW) <= kSelKeys;
+  // (the limit of shared memory is the same for every call: other threads set it too)
+  constexpr int kSelMaxSmem = 4 * (kSelHist + kSelKeys);
+  const bool cluster = nnz > 0 && select_keys(N, SW) <= kSelKeys &&
+                       clusters_at_once<tern_select_kernel>(kSelCtas, kSelThreads, kSelMaxSmem) > 0;
   cudaError_t e = cudaSuccess;
   if (nnz == 0) e = cudaMemsetAsync(sal, 0, (size_t)NW * 4, s);
   if (nnz > 0 && !cluster) e = cudaMemsetAsync(sw, 0, sizeof(SelWork), s);
@@ -738,12 +743,10 @@ cudaError_t launch_ternarize(int N, int K, const uint16_t *W, int64_t nnz, int s
   tern_stats_kernel<<<grid_blocks(NB), kBlockThreads, 0, s>>>(NB, W, stats, keys, status);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if (cluster) {
-    // (the limit does not depend on the call: other threads set it too)
     const int smem = (int)(4 * (kSelHist + select_keys(N, SW)));
     e = cudaFuncSetAttribute(tern_select_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(tern_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             4 * (kSelHist + kSelKeys));
+    e = cudaFuncSetAttribute(tern_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSelMaxSmem);
     if (e != cudaSuccess) return e;
     e = launch_dependent_cluster(tern_select_kernel, dim3(kSelCtas), kSelCtas, kSelThreads, smem, s, N, G, SW,
                                  (uint32_t)nnz, keys, sal, rowptr);

@@ -101,3 +101,14 @@ def test_prefill_splits_only_where_clusters_run(launches):
     assert no == [0, [1], 0]
     assert failed == [0, [1], 0]  # the query's error is not the call's
     assert launches((0, -1, call)) == [[0, [1], 0]]
+
+
+def test_ternarize_selects_without_a_cluster(launches):
+    """Statistics, selection, planes: one cluster of 16 where the device holds
+    one, else the whole chip's kernels (four digits, count, mark, rowptr)."""
+    call = ("ternarize", 256, 1024, 200)
+    (one, no, failed, other) = launches((0, 1, call), (1, 0, call), (2, -1, call), (3, 1, call))
+    assert one == [0, [1, 16, 1], 0] and other == [0, [1, 16, 1], 0]
+    assert no == [0, [1] * 9, 0] and failed == [0, [1] * 9, 0]
+    too_many = ("ternarize", 26609, 128, 200)  # keys beyond the cluster's shared memory
+    assert launches((0, 1, too_many)) == [[0, [1] * 9, 0]]

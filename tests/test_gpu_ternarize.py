@@ -4,6 +4,8 @@ sides take every decision in IEEE float32 with sums in index order); the
 fp16 offsets and scales within one fp16 unit in the last place (the GPU runs
 the refinement sweeps on each block's moments, the oracle in passes over the
 weights: the same updates, rounded differently in float32)."""
+import os
+
 import numpy as np
 import pytest
 import torch
@@ -116,6 +118,44 @@ def test_ternarize_selection_paths(N, K, frac):
     W[b % 5 < 2] = W[b % 5 < 2, :1]
     W = W.reshape(N, K)
     compare(W, int(round(frac * len(b))), 2)
+
+
+NO_CLUSTERS = r"""
+int cudaOccupancyMaxActiveClusters(int *n, const void *f, const void *c) { *n = 0; return 0; }
+"""
+SELECT_SHAPES = [(1, 128, 1.0), (15, 33 * 128, 0.1), (37, 384, 0.1), (300, 2560, 0.1), (97, 640, 1.0), (4096, 1024, 0.3)]
+SELECT_ALL = r"""
+import sys
+sys.path[:0] = [sys.argv[1], sys.argv[1] + "/tests"]
+import torch
+import test_gpu_ternarize as t
+torch.save(t.select_all(), sys.argv[2])
+"""
+
+
+def select_all():
+    from paper_2609_09240_gb300 import tq
+    out = []
+    for N, K, frac in SELECT_SHAPES:
+        W = torch.from_numpy(wl.gen_dense_weights(N, K, config=9, proj=5).view(np.float16)).cuda()
+        w = tq.ternarize(W, int(round(frac * N * (K // 128))), index=False)
+        out += [t.cpu() for t in (w.plane1, w.salience, w.rowptr, w.plane2, w.scale1, w.offset, w.scale2)]
+    return out
+
+
+def test_ternarize_selection_without_clusters(tmp_path):
+    """A process whose device reports room for no cluster selects over the
+    whole chip at every size: the same bytes."""
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    (tmp_path / "none.c").write_text(NO_CLUSTERS)
+    subprocess.run(["gcc", "-shared", "-fPIC", "-o", str(tmp_path / "none.so"), str(tmp_path / "none.c")], check=True)
+    r = subprocess.run([sys.executable, "-c", SELECT_ALL, root, str(tmp_path / "out.pt")], capture_output=True, text=True,
+                       env=dict(os.environ, LD_PRELOAD=str(tmp_path / "none.so")))
+    assert r.returncode == 0, r.stderr
+    for a, b in zip(torch.load(tmp_path / "out.pt"), select_all()):
+        assert torch.equal(a.view(torch.uint8), b.view(torch.uint8))
 
 
 def test_ternarize_full_size_gate_projection():
