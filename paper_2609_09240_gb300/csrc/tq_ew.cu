@@ -16,6 +16,7 @@
 #include <type_traits>
 
 #include "tq_common.cuh"
+#include "tq_ew_pairs.cuh"
 #include "tq_launch.cuh"
 #include "tq_sm100.cuh"
 
@@ -417,11 +418,15 @@ __global__ void __launch_bounds__(kIdxThreads, MT == 8 ? 1 : 2)
     grid_dep_wait();  // the plane-1 pass (returns at once from the second time on)
     const int r_lo = b_lo + (b_hi - b_lo) * warp / kIdxWarps, r_hi = b_lo + (b_hi - b_lo) * (warp + 1) / kIdxWarps;
     if (r_lo >= r_hi) continue;
-    // entries as aligned pairs: entry i is half (i + odd) & 1 of word (i + odd) / 2
+    // entries as aligned pairs, but for the index's first and last where a word
+    // of theirs reaches beyond it (tq_ew_pairs.cuh): their rows add them alone
     const int odd = (int)(((uintptr_t)w.idx >> 1) & 1u);
     const uint32_t *iw = reinterpret_cast<const uint32_t *>(w.idx - odd);
     const int32_t *offs = w.idx_off + (int64_t)r_lo * nb;
-    const int blocks = (r_hi - r_lo) * nb;
+    const int blocks = (r_hi - r_lo) * nb, entries = __ldg(w.idx_off + (int64_t)N * nb), last = pairs_end(odd, entries);
+    const bool alone = (read_alone(false, odd, entries) && __ldg(offs) == 0) ||
+                       (read_alone(true, odd, entries) && __ldg(offs + blocks) == entries);
+    auto off_at = [&](int i) { return pairs_clamp(__ldg(offs + i), odd, last); };
     auto load_pairs = [&](uint32_t (&v)[kIdxAhead], int e, int e1) {
       const int first = (e + odd) >> 1, c = ((e1 + odd + 1) >> 1) - first;
       const uint32_t *q = iw + first + lane;
@@ -439,8 +444,8 @@ __global__ void __launch_bounds__(kIdxThreads, MT == 8 ? 1 : 2)
     };
     auto h2f = [](unsigned short v) { return __half2float(__ushort_as_half(v)); };
     load_params(r_lo);
-    int e = __ldg(offs), e1 = __ldg(offs + 1);
-    int e2 = blocks > 1 ? __ldg(offs + 2) : e1;  // the next block's end
+    int e = off_at(0), e1 = off_at(1);
+    int e2 = blocks > 1 ? off_at(2) : e1;  // the next block's end
     uint32_t v[kIdxAhead];
     load_pairs(v, e, e1);
     int f = 0;  // the block among the run's
@@ -456,29 +461,28 @@ __global__ void __launch_bounds__(kIdxThreads, MT == 8 ? 1 : 2)
       float acc[MT];
 #pragma unroll
       for (int t = 0; t < MT; ++t) acc[t] = 0.f;
+      auto add_at = [&](uint32_t en, bool in, int b) {  // en: the entry (of block b) in bits 0..15
+        if constexpr (STAGED) {
+          const float wt = lds_f32((en >> 9 & 0x7cu) | tab_a);
+          float x[MT];
+          staged_acts<MT>((en << kESLog & ((kIdxBlock - 1) << kESLog)) | (xs_a + (uint32_t)b * kBlockBytes), x);
+          if (in) {
+#pragma unroll
+            for (int t = 0; t < MT; ++t) acc[t] = fmaf(wt, x[t], acc[t]);
+          }
+        } else if (in) {
+          const float wt = tab[en >> kIdxShift & 31u];
+          const int k = min(b * kIdxBlock + (int)(en & (kIdxBlock - 1)), K - 1);
+#pragma unroll
+          for (int t = 0; t < MT; ++t)
+            if (t < mt) acc[t] = fmaf(wt, h2f(__ldg(xm + (int64_t)t * K + k)), acc[t]);
+        }
+      };
       for (int b = 0; b < nb; ++b, ++f) {
-        const int e3 = f + 2 < blocks ? __ldg(offs + f + 3) : e2;
+        const int e3 = f + 2 < blocks ? off_at(f + 3) : e2;
         uint32_t u[kIdxAhead];  // the next block's entries
         load_pairs(u, e1, e2);
-        const uint32_t xb = xs_a + (uint32_t)b * kBlockBytes;
-        const int kb = b * kIdxBlock, kmax = K - 1 - kb;
-        auto add = [&](uint32_t en, bool in) {  // en: the entry in bits 0..15
-          if constexpr (STAGED) {
-            const float wt = lds_f32((en >> 9 & 0x7cu) | tab_a);
-            float x[MT];
-            staged_acts<MT>((en << kESLog & ((kIdxBlock - 1) << kESLog)) | xb, x);
-            if (in) {
-#pragma unroll
-              for (int t = 0; t < MT; ++t) acc[t] = fmaf(wt, x[t], acc[t]);
-            }
-          } else if (in) {
-            const float wt = tab[en >> kIdxShift & 31u];
-            const int k = kb + min((int)(en & (kIdxBlock - 1)), kmax);
-#pragma unroll
-            for (int t = 0; t < MT; ++t)
-              if (t < mt) acc[t] = fmaf(wt, h2f(__ldg(xm + (int64_t)t * K + k)), acc[t]);
-          }
-        };
+        auto add = [&](uint32_t en, bool in) { add_at(en, in, b); };
         const int front = (e + odd) & 1, c = e1 - e + front;  // entries from the first word on, the first `front` not ours
 #pragma unroll
         for (int j = 0; j < kIdxAhead; ++j) {
@@ -494,6 +498,16 @@ __global__ void __launch_bounds__(kIdxThreads, MT == 8 ? 1 : 2)
         e = e1, e1 = e2, e2 = e3;
 #pragma unroll
         for (int j = 0; j < kIdxAhead; ++j) v[j] = u[j];
+      }
+      if (alone) {
+        const int32_t *ro = offs + (int64_t)(n - r_lo) * nb;
+        for (int side = 0; side < 2; ++side) {
+          const int i = side ? entries - 1 : 0;
+          if (!read_alone(side, odd, entries) || i < __ldg(ro) || i >= __ldg(ro + nb)) continue;
+          int b = 0;  // the entry's block
+          while (__ldg(ro + b + 1) <= i) ++b;
+          add_at(__ldg(w.idx + i), lane == 0, b);
+        }
       }
       float mine = 0.f;
 #pragma unroll

@@ -302,3 +302,44 @@ def test_linear_indexed_odd_index_address(H, M, N, K):
     for out in (y, tq.tq_ew_linear(x, g)):
         H.device_status_ok()
         H.assert_close(out.float().cpu().numpy().astype(np.float64), y_ref, a_ref)
+
+
+@pytest.mark.parametrize("odd", [0, 1])
+@pytest.mark.parametrize("parity", [0, 1])
+@pytest.mark.parametrize("M,N,K,lead,tail", [
+    (1, 5, 128, 0, 0), (4, 40, 4096, 3, 2), (1, 300, 2176, 0, 17), (8, 7, 256, 6, 0),
+    (1, 3, 131072, 1, 0), (5, 3, 131072, 0, 1),  # x from global memory
+])
+def test_linear_indexed_first_and_last_entry(H, M, N, K, lead, tail, odd, parity):
+    """The index's first and last entries (their weights 64 among weights of
+    about 0.02, behind `lead` and before `tail` empty rows) at both alignments
+    and with an even and an odd number of entries."""
+    from paper_2609_09240_gb300 import tq
+    w = wl.gen_ew_weights(N, K, config=27, proj=M + N)
+    w.mask[w.mask == 0] = 1
+    w.mask[:lead] = 3
+    w.mask[N - tail:] = 3
+    ends = [(lead, K // 3), (N - 1 - tail, K // 2)]
+    w.mask[ends[0][0], :ends[0][1]] = 3
+    w.mask[ends[1][0], ends[1][1]:] = 3
+    for n, k in ends:
+        w.mask[n, k], w.T0[n, k] = 0, 1
+    if (np.count_nonzero(w.mask < 3) - parity) % 2:  # one entry between them more or fewer
+        n, k = ends[0][0], ends[0][1] + 1
+        w.mask[n, k] = 2 if w.mask[n, k] == 3 else 3
+    w.T1[w.mask >= 2] = 0
+    w.a0.view(np.float16)[:, 0] = 64.0
+    x = wl.gen_x(M, K, config=27, proj=M + N)
+    g = _indexed(H, w)
+    entries = int(g.idx_off[-1].item())
+    assert entries % 2 == parity
+    moved = torch.zeros(entries + odd, dtype=g.idx.dtype, device="cuda")
+    moved[odd:] = g.idx[:entries]
+    g.idx = moved[odd:]
+    assert g.idx.data_ptr() % 4 == 2 * odd
+    mp, p1, rp, p2, st = ew.pack(w.T0, w.T1, w.mask)
+    assert st == 0
+    y_ref, a_ref = ew.linear(x, K, mp, p1, rp, p2, w.mu, w.a0, w.a1)
+    y = tq.tq_ew_linear(H.dev(x), g)
+    H.device_status_ok()
+    H.assert_close(y.float().cpu().numpy().astype(np.float64), y_ref, a_ref)
