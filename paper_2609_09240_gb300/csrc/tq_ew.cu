@@ -358,9 +358,15 @@ __device__ __forceinline__ void staged_acts(uint32_t a, float (&x)[MT]) {
 // is 8 us), against 31.6 M in 39.5 us with one guarded entry per lane and
 // step, and 48 us with gathers from global memory.
 // STAGED = false reads x from global memory: K x tokens beyond a block's
-// shared memory.
+// shared memory.  What binds is then the latency of the gathers, so a lane has
+// ten under way (each loaded whether or not its entry is one), and one or two
+// tokens take 64 registers, so that an SM holds 32 warps, since a long call is
+// faster for it (16384 x 57344, one token, 13.6 and 60 % coverage: 212 and
+// 683 us, with 128 registers 234 and 1018, with a gather at a time for eight
+// tokens, whatever the call's, 625 and 2712, from warps of a row each 285 and
+// 725; 300 x 57344 with 13.6 %: 38, 34, 91 and 79).
 template <bool F32, int MT, bool STAGED, class BT>
-__global__ void __launch_bounds__(kIdxThreads, MT == 8 ? 1 : 2)
+__global__ void __launch_bounds__(kIdxThreads, MT == 8 || (!STAGED && MT > 2) ? 1 : 2)
     correct_idx_kernel(const __grid_constant__ BT bt, int64_t total, int m0, int mt) {
   constexpr int kES = elem_bytes(MT), kBlockBytes = kIdxBlock * kES;
   constexpr int kESLog = MT == 8 ? 4 : MT == 4 ? 3 : 2;
@@ -470,12 +476,18 @@ __global__ void __launch_bounds__(kIdxThreads, MT == 8 ? 1 : 2)
 #pragma unroll
             for (int t = 0; t < MT; ++t) acc[t] = fmaf(wt, x[t], acc[t]);
           }
-        } else if (in) {
+        } else {
+          // (loaded whether or not `in`: the gathers of a lane's entries are
+          // then under way together)
           const float wt = tab[en >> kIdxShift & 31u];
-          const int k = min(b * kIdxBlock + (int)(en & (kIdxBlock - 1)), K - 1);
+          const unsigned short *xk = xm + min(b * kIdxBlock + (int)(en & (kIdxBlock - 1)), K - 1);
+          unsigned short x[MT];
 #pragma unroll
-          for (int t = 0; t < MT; ++t)
-            if (t < mt) acc[t] = fmaf(wt, h2f(__ldg(xm + (int64_t)t * K + k)), acc[t]);
+          for (int t = 0; t < MT; ++t) x[t] = __ldg(xk + (int64_t)min(t, mt - 1) * K);
+          if (in) {
+#pragma unroll
+            for (int t = 0; t < MT; ++t) acc[t] = fmaf(wt, h2f(x[t]), acc[t]);
+          }
         }
       };
       for (int b = 0; b < nb; ++b, ++f) {
@@ -484,16 +496,35 @@ __global__ void __launch_bounds__(kIdxThreads, MT == 8 ? 1 : 2)
         load_pairs(u, e1, e2);
         auto add = [&](uint32_t en, bool in) { add_at(en, in, b); };
         const int front = (e + odd) & 1, c = e1 - e + front;  // entries from the first word on, the first `front` not ours
+        const int i0 = 2 * lane;
+        add(v[0], i0 < c && i0 >= front);
+        add(v[0] >> 16, i0 + 1 < c);
+        if (STAGED || c > 64) {  // (a block of few entries gathers for these only)
 #pragma unroll
-        for (int j = 0; j < kIdxAhead; ++j) {
-          const int i = 2 * (lane + 32 * j);
-          add(v[j], j == 0 ? i < c && i >= front : i < c);
-          add(v[j] >> 16, i + 1 < c);
+          for (int j = 1; j < kIdxAhead; ++j) {
+            const int i = i0 + 64 * j;
+            add(v[j], i < c);
+            add(v[j] >> 16, i + 1 < c);
+          }
         }
-        for (int i = 2 * (lane + 32 * kIdxAhead); i < c; i += 64) {
-          const uint32_t r = __ldg(iw + ((e + odd) >> 1) + (i >> 1));
-          add(r, true);
-          add(r >> 16, i + 1 < c);
+        if constexpr (STAGED) {
+          for (int i = 2 * (lane + 32 * kIdxAhead); i < c; i += 64) {
+            const uint32_t r = __ldg(iw + ((e + odd) >> 1) + (i >> 1));
+            add(r, true);
+            add(r >> 16, i + 1 < c);
+          }
+        } else {  // as many gathers under way as for the first entries
+          for (int i1 = i0 + 64 * kIdxAhead; i1 - i0 < c; i1 += 64 * kIdxAhead) {
+            uint32_t r[kIdxAhead];
+#pragma unroll
+            for (int j = 0; j < kIdxAhead; ++j)
+              r[j] = i1 + 64 * j < c ? __ldg(iw + ((e + odd) >> 1) + (i1 >> 1) + 32 * j) : 0u;
+#pragma unroll
+            for (int j = 0; j < kIdxAhead; ++j) {
+              add(r[j], i1 + 64 * j < c);
+              add(r[j] >> 16, i1 + 64 * j + 1 < c);
+            }
+          }
         }
         e = e1, e1 = e2, e2 = e3;
 #pragma unroll
@@ -549,14 +580,16 @@ cudaError_t launch_correct(int M, const Batch<Prob> &bt, int grid, cudaStream_t 
   return cudaSuccess;
 }
 
-// grid: blocks for the call's indexed rows at one row per warp, capped at
-// what the chip holds.
+// grid: blocks for the call's indexed rows at one row per warp (at two warps
+// per row where x is gathered: few rows are then on more SMs), capped at what
+// the chip holds.
 template <bool F32, int MT, bool STAGED>
 cudaError_t launch_correct_idx(int M, const Batch<Prob> &bt, int64_t total, int rows, int Kmax, int num_sms,
                                cudaStream_t s) {
   const int smem = STAGED ? (int)idx_smem_bytes(Kmax, MT) : kIdxTabBytes;
-  const int per_sm = MT < 8 && 2 * (smem + 1024) <= kSmSmem ? 2 : 1;
-  const int grid = std::max(1, std::min((rows + kIdxWarps - 1) / kIdxWarps, per_sm * num_sms));
+  const int per_sm = MT < 8 && (STAGED || MT <= 2) && 2 * (smem + 1024) <= kSmSmem ? 2 : 1;
+  constexpr int kRowsPerBlock = STAGED ? kIdxWarps : kIdxWarps / 2;
+  const int grid = std::max(1, std::min((rows + kRowsPerBlock - 1) / kRowsPerBlock, per_sm * num_sms));
   return with_batch(bt, [&](const auto &b) {
     const auto kern = correct_idx_kernel<F32, MT, STAGED, std::decay_t<decltype(b)>>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kIdxMaxSmem);
@@ -575,16 +608,23 @@ cudaError_t launch_correct_mt(int M, const Batch<Prob> &bt, int grid, cudaStream
 }
 
 // Tokens per pass: as many as the call has, up to 8, while their staged
-// activations fit a block's shared memory (K up to 12288 for 8 tokens,
-// 55296 for one); beyond that x is gathered from global memory.
+// activations fit a block's shared memory (K up to 12288 for 8 tokens, 26624
+// for four, 55296 for two or one); beyond that x is gathered from global
+// memory.  More passes than three of two tokens each are slower than one of
+// eight that gathers (512 x 49152, eight tokens, 13.6 %: 150 and 141 us, with
+// 0.3 % 148 and 107); with passes of four, staging is the faster one
+// (4096 x 16384, eight tokens: 65 and 77, but 62 and 50 with 0.3 %).
 template <bool F32>
 cudaError_t launch_correct_idx_mt(int M, const Batch<Prob> &bt, int64_t total, int rows, int Kmax, int num_sms,
                                   cudaStream_t s) {
   const auto fits = [&](int MT) { return idx_smem_bytes(Kmax, MT) <= kIdxMaxSmem; };
   if (M > 4 && fits(8)) return launch_correct_idx<F32, 8, true>(M, bt, total, rows, Kmax, num_sms, s);
   if (M > 2 && fits(4)) return launch_correct_idx<F32, 4, true>(M, bt, total, rows, Kmax, num_sms, s);
-  if (M > 1 && fits(2)) return launch_correct_idx<F32, 2, true>(M, bt, total, rows, Kmax, num_sms, s);
+  if (M > 1 && M <= 6 && fits(2)) return launch_correct_idx<F32, 2, true>(M, bt, total, rows, Kmax, num_sms, s);
   if (M == 1 && fits(1)) return launch_correct_idx<F32, 1, true>(M, bt, total, rows, Kmax, num_sms, s);
+  if (M == 1) return launch_correct_idx<F32, 1, false>(M, bt, total, rows, Kmax, num_sms, s);
+  if (M == 2) return launch_correct_idx<F32, 2, false>(M, bt, total, rows, Kmax, num_sms, s);
+  if (M <= 4) return launch_correct_idx<F32, 4, false>(M, bt, total, rows, Kmax, num_sms, s);
   return launch_correct_idx<F32, 8, false>(M, bt, total, rows, Kmax, num_sms, s);
 }
 

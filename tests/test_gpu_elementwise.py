@@ -343,3 +343,24 @@ def test_linear_indexed_first_and_last_entry(H, M, N, K, lead, tail, odd, parity
     y = tq.tq_ew_linear(H.dev(x), g)
     H.device_status_ok()
     H.assert_close(y.float().cpu().numpy().astype(np.float64), y_ref, a_ref)
+
+
+@pytest.mark.parametrize("M,N,K,cover", [
+    (1, 20, 57344, (0.3, 0.3, 0.3)),        # x from global memory: full blocks, and rows that share a block of warps
+    (2, 9, 65536, (0.3, 0.3, 0.4)),
+    (3, 5, 65536, (0.005, 0.01, 0.01)),     # a block's entries in a lane's first word
+    (4, 7, 57472, (0.2, 0.2, 0.2)),         # a last block of 128
+    (6, 9, 32768, (0.005, 0.031, 0.10)),    # three passes of two tokens
+    (7, 9, 32768, (0.3, 0.3, 0.3)),         # one of eight
+    (12, 5, 28672, (0.001, 0.001, 0.001)),
+])
+def test_linear_indexed_long_rows(H, M, N, K, cover):
+    from paper_2609_09240_gb300 import tq
+    w = wl.gen_ew_weights(N, K, config=28, proj=M + N, coverage=cover)
+    xb = wl.gen_x(M, K, config=28, proj=M + N)
+    mp, p1, rp, p2, st = ew.pack(w.T0, w.T1, w.mask)
+    assert st == 0
+    y_ref, a_ref = ew.linear(xb, K, mp, p1, rp, p2, w.mu, w.a0, w.a1)
+    y = tq.tq_ew_linear(H.dev(xb), _indexed(H, w), f32=True)
+    H.device_status_ok()
+    H.assert_close(y.cpu().numpy().astype(np.float64), y_ref, a_ref)
