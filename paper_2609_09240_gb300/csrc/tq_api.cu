@@ -8,7 +8,7 @@
 #include "tq_common.cuh"
 
 namespace tq {
-cudaError_t launch_rowptr(int N, int K, const uint32_t *sal, int32_t *rowptr, uint32_t *status,
+cudaError_t launch_rowptr(int N, int K, const uint32_t *sal, int32_t *rowptr, uint32_t *status, bool behind_smem,
                           cudaStream_t s);
 cudaError_t launch_pack(int N, int K, const int8_t *T1, const int8_t *T2, const uint32_t *sal,
                         const int32_t *rowptr, uint8_t *plane1, uint8_t *plane2, uint32_t *status,
@@ -230,7 +230,7 @@ tq_status tq_salience_rowptr(int32_t N, int32_t K, const uint32_t *sal, int32_t 
                              uint32_t *d_status, void *stream) {
   if (tq_status st = check_shape(N, K)) return st;
   if (!sal || !rowptr || !d_status) return TQ_ERR_NULL;
-  return from_cuda(launch_rowptr(N, K, sal, rowptr, d_status, (cudaStream_t)stream));
+  return from_cuda(launch_rowptr(N, K, sal, rowptr, d_status, false, (cudaStream_t)stream));
 }
 
 tq_status tq_pack(int32_t N, int32_t K, const int8_t *T1, const int8_t *T2, const uint32_t *sal,

@@ -694,8 +694,17 @@ static int grid_for(int64_t work, int block) {
   return (int)(g < 1 ? 1 : g);
 }
 
-cudaError_t launch_rowptr(int N, int K, const uint32_t *sal, int32_t *rowptr, uint32_t *status,
+// behind_smem: the stream's previous kernel may be one whose CTAs fill shared
+// memory.  Beside them this one gets little of the SM's L1 cache, on which its
+// strided reads live where a thread has more than 16 rows, so it then waits
+// for their end: ternarizing 40000 x 128 took 92 us with an early start and
+// takes 66 without (10 % salient 129 and 96).
+cudaError_t launch_rowptr(int N, int K, const uint32_t *sal, int32_t *rowptr, uint32_t *status, bool behind_smem,
                           cudaStream_t s) {
+  if (behind_smem && N > 16 * 1024) {
+    rowptr_kernel<<<1, 1024, 0, s>>>(N, K, sal, rowptr, status);
+    return cudaGetLastError();
+  }
   return launch_dependent(rowptr_kernel, dim3(1), 1024, s, N, K, sal, rowptr, status);
 }
 

@@ -38,7 +38,8 @@
 //                       the packed bytes and fp16 parameters (salient blocks
 //                       by record, in CTAs of their own).
 // Each is launched while its predecessor still runs (programmatic dependent
-// launch) and waits for it before it reads anything.
+// launch) and waits for it before it reads anything (rowptr of many rows, after
+// its end).
 #include <algorithm>
 
 #include "tq_common.cuh"
@@ -47,7 +48,7 @@
 
 namespace tq {
 
-cudaError_t launch_rowptr(int N, int K, const uint32_t *sal, int32_t *rowptr, uint32_t *status,
+cudaError_t launch_rowptr(int N, int K, const uint32_t *sal, int32_t *rowptr, uint32_t *status, bool behind_smem,
                           cudaStream_t s);
 
 namespace tz {
@@ -765,7 +766,7 @@ cudaError_t launch_ternarize(int N, int K, const uint16_t *W, int64_t nnz, int s
           cudaSuccess)
         return e;
     }
-    if ((e = launch_rowptr(N, K, sal, rowptr, status, s)) != cudaSuccess) return e;
+    if ((e = launch_rowptr(N, K, sal, rowptr, status, true, s)) != cudaSuccess) return e;
   }
   __half *h1 = reinterpret_cast<__half *>(scale1), *ho = reinterpret_cast<__half *>(offset);
   const int p2 = nnz > 0 ? grid_blocks(nnz) : 0;
