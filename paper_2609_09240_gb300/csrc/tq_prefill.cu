@@ -598,7 +598,12 @@ static cudaError_t launch_prefill_group(const Problem *probs, int count, int M, 
   }
   // CTAs per tile: the most whose clusters all run at once (more would wait
   // for the first to end: 16 clusters of eight for 512 tokens x 1024 x 2560
-  // took 29.2 us, of four 18.5), two groups each at least
+  // took 29.2 us, of four 18.5), two groups each at least.  Exchanging the
+  // partial sums takes as long as five or six groups, more on a full chip, so
+  // a tile is shared where each CTA saves that many (10 % salient: 256 tokens x
+  // 640 x 512, two groups of four saved, 15.4 us shared and 11.3 alone; 128 x
+  // 1024 x 1024, six of eight, 14.6 and 16.5; 512 x 4096 x 1280, five of ten on
+  // 128 SMs, 20.5 and 19.5).
   int split = 1;
   int gmin = probs[0].K / kGroup;
   for (int i = 1; i < count; ++i) gmin = std::min(gmin, probs[i].K / kGroup);
@@ -607,6 +612,7 @@ static cudaError_t launch_prefill_group(const Problem *probs, int count, int M, 
     return clusters_at_once<pf::prefill2_kernel<false, 1, true>>(c, pf::kThreads2, pf::Lay2<1>::kSmem);
   };
   while (!wide && 2 * split <= pf::kMaxSplit && gmin >= 4 * split && tiles <= at_once(2 * split)) split *= 2;
+  if (gmin - (gmin + split - 1) / split < (split * tiles > sms / 2 ? 7 : 6)) split = 1;
   if (split > 1) {
     auto kern = f32 ? pf::prefill2_kernel<true, 1, true> : pf::prefill2_kernel<false, 1, true>;
     const int smem = pf::Lay2<1>::kSmem;

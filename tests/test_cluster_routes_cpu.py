@@ -29,6 +29,10 @@ int cudaMemsetAsync(void *p, int v, size_t n, void *s) { return 0; }
 int cudaOccupancyMaxActiveClusters(int *n, const void *f, const cfg_ *c) {
   if (clusters[device] < 0) return fail(1);
   *n = clusters[device];
+  if (*n == 999) {  /* a whole chip's counts */
+    const int size = (int)c->attrs[0].val.d.x;
+    *n = size == 2 ? 76 : size == 4 ? 36 : size == 8 ? 15 : 1;
+  }
   return 0;
 }
 int cudaLaunchKernelExC(const cfg_ *c, const void *f, void **args) {
@@ -101,6 +105,15 @@ def test_prefill_splits_only_where_clusters_run(launches):
     assert no == [0, [1], 0]
     assert failed == [0, [1], 0]  # the query's error is not the call's
     assert launches((0, -1, call)) == [[0, [1], 0]]
+
+
+def test_prefill_splits_only_where_it_saves_groups(launches):
+    shapes = [((256, 640, 512), 1), ((256, 640, 896), 1),   # two and three groups saved
+              ((128, 1024, 1024), 4), ((128, 1024, 2048), 8),
+              ((512, 4096, 1280), 1), ((512, 4096, 1536), 1), ((512, 4096, 1792), 2),  # 64 tiles
+              ((200, 9728, 2560), 2), ((200, 19456, 2560), 1)]
+    got = launches(*[(0, 999, ("prefill", *shape)) for shape, _ in shapes])
+    assert got == [[0, [split], 0] for _, split in shapes]
 
 
 def test_ternarize_selects_without_a_cluster(launches):

@@ -409,3 +409,23 @@ def test_prefill_shared_tiles(H, M, shapes, frac, f32):
     H.device_status_ok()
     for y, (y_ref, a_ref) in zip(ys, refs):
         H.assert_close(y.float().cpu().numpy().astype(np.float64), y_ref, a_ref)
+
+
+@pytest.mark.parametrize("M,N,K", [
+    (200, 1000, 8448),   # eight CTAs, 66 groups: shares that begin in the second and third salience word
+    (40, 300, 2048),     # eight CTAs of two groups
+    (129, 1025, 1152),   # four CTAs of two and three groups
+    (256, 9728, 1792),   # two CTAs for every SM
+    (300, 640, 896),     # too few groups saved: a CTA per tile
+])
+@pytest.mark.parametrize("frac", [0.0, 0.3, 1.0])
+@pytest.mark.parametrize("f32", [False, True])
+def test_prefill_shares_by_output_type(H, M, N, K, frac, f32):
+    from paper_2609_09240_gb300 import tq
+    w = wl.gen_weights(N, K, frac, config=6, proj=90)
+    x = wl.gen_x(M, K, config=6, proj=90)
+    rows = np.sort(np.random.default_rng(N).choice(N, size=min(N, 200), replace=False)).astype(np.int32)
+    y_ref, a_ref = H.oracle_ref(w, x, rows=rows)
+    y = (tq.tq_linear_f32out if f32 else tq.tq_linear)(H.dev(x), H.pack_on_gpu(w))
+    H.device_status_ok()
+    H.assert_close(y.float().cpu().numpy()[:, rows].astype(np.float64), y_ref, a_ref)
