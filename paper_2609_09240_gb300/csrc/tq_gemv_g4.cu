@@ -609,11 +609,13 @@ __device__ __forceinline__ int unit_parts(int K, int SG, int split) {
 // second-plane warps have their first tiles' group, operands and records in
 // registers when the barrier opens, the decode warps the next problem's
 // parameters and walk (worked out from a cold parameter space after the
-// barrier they took 3500 cycles a problem), and a row of y is loaded after the
-// barrier and stored after the next problem's stages.  One Qwen3-8B step of
-// 144 problems: 1.14 ms; with the second plane done by the decode warps before
-// their stages, and all of this after the barrier, 1.61.  barrier_extra > 0 makes every barrier wait for CTAs that do not
-// exist, so that its bounded wait runs out (the failure-path self-test).
+// barrier they took 3500 cycles a problem).  y is stored before the next
+// problem's stages: holding a row of it until after them took 1.136 ms per
+// Qwen3-8B step of 144 problems instead of 1.117 (and the registers for it
+// spilled); with the second plane done by the decode warps before their
+// stages, and all of this after the barrier, 1.61.  barrier_extra > 0 makes
+// every barrier wait for CTAs that do not exist, so that its bounded wait runs
+// out (the failure-path self-test).
 struct SeqWalk {
   const BatchParams *bp;
   int cta, ctas, p, unit, u_end, u, nst, tile, s, s_end;
@@ -766,12 +768,7 @@ __global__ void __launch_bounds__((kWD1 + 1 + kSeqP2) * 32, 1)
     uint32_t bz[kBSets][4] = {};
     uint32_t buf = 0, phase = 0;
     SeqWalk w(&bp, blockIdx.x, gridDim.x);
-    // rows [r0, r1) of a finished problem whose y this CTA stores; the
-    // thread's first row waits in yv
-    void *yp = nullptr;
-    int r0 = 0, r1 = 0;
-    float yv = 0.f;
-    auto y_store = [&](int n, float v) {
+    auto y_store = [&](void *yp, int n, float v) {
       if (F32)
         static_cast<float *>(yp)[n] = v;
       else
@@ -800,7 +797,6 @@ __global__ void __launch_bounds__((kWD1 + 1 + kSeqP2) * 32, 1)
         if (++buf == (uint32_t)kNS) buf = 0, phase ^= 1u;
       }
       if constexpr (ONE) break;
-      if (r0 + tid < r1) y_store(r0 + tid, yv);  // of the problem before
       // the problem's barrier: every CTA's additions into y2 are done
       if (warp != 0) {
         named_bar_arrive(1, kWorkers);
@@ -815,8 +811,8 @@ __global__ void __launch_bounds__((kWD1 + 1 + kSeqP2) * 32, 1)
       // what the next problem needs of the parameters, while the others finish
       const int target = (w.p + 1) * ((int)gridDim.x + barrier_extra);
       const float *y2 = P.y2();
-      yp = P.y;
-      r0 = share_at(P.N, blockIdx.x, gridDim.x), r1 = share_at(P.N, blockIdx.x + 1, gridDim.x);
+      void *const yp = P.y;
+      const int r0 = share_at(P.N, blockIdx.x, gridDim.x), r1 = share_at(P.N, blockIdx.x + 1, gridDim.x);
       more = w.next_problem();
       if (warp == 0 && lane == 0 && ok && !*abort_) {
         const uint64_t t0 = global_ns();
@@ -833,14 +829,9 @@ __global__ void __launch_bounds__((kWD1 + 1 + kSeqP2) * 32, 1)
       __syncwarp();
       // stop together: the flag may be raised (by the producer) while
       // the warps read it, so they decide by one reduction over the barrier
-      if (named_bar_any(2, kWorkers, *abort_ != 0)) {
-        r1 = 0;
-        break;
-      }
-      // this CTA's slice of the problem's output: the thread's first row is
-      // loaded here and stored after the next problem's stages
-      if (r0 + tid < r1) yv = __ldcg(y2 + r0 + tid);
-      for (int n = r0 + tid + WD * 32; n < r1; n += WD * 32) y_store(n, __ldcg(y2 + n));
+      if (named_bar_any(2, kWorkers, *abort_ != 0)) break;
+      // this CTA's slice of the problem's output
+      for (int n = r0 + tid; n < r1; n += WD * 32) y_store(yp, n, __ldcg(y2 + n));
     }
     if constexpr (ONE) {
       named_bar(1, kWorkers);
@@ -853,7 +844,6 @@ __global__ void __launch_bounds__((kWD1 + 1 + kSeqP2) * 32, 1)
       if (named_bar_any(2, WD * 32, last)) {
         const Problem &P = bp.prob[0];
         const float *y2 = P.y2();
-        yp = P.y;
         constexpr int B = 16;  // rows a thread has in flight
         for (int n0 = tid; n0 < P.N; n0 += B * WD * 32) {
           float v[B];
@@ -865,12 +855,10 @@ __global__ void __launch_bounds__((kWD1 + 1 + kSeqP2) * 32, 1)
 #pragma unroll
           for (int i = 0; i < B; ++i) {
             const int n = n0 + i * WD * 32;
-            if (n < P.N) y_store(n, v[i]);
+            if (n < P.N) y_store(P.y, n, v[i]);
           }
         }
       }
-    } else if (r0 + tid < r1) {
-      y_store(r0 + tid, yv);
     }
   } else if (warp == WD) {
     // ========================================================== producer
