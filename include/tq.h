@@ -335,10 +335,10 @@ TQ_API tq_status tq_linear_batched(int32_t M, int32_t count, const tq_problem *p
  * runtime runs one token's layers in order).  Like tq_linear_batched, but
  * problem i + 1 starts only once problem i has completed on every SM (the
  * sums of all its rows are complete; each SM stores its share of y_i before
- * it goes on to problem i + 1), as the layers of a model need: e.g. per layer q/k/v (rows concatenated into
- * one weight), o, gate/up (concatenated), down.  The attention, norms and
- * activation between them are outside this library: every problem's x is
- * an input of the call.  One persistent launch after the activation prep;
+ * it goes on to problem i + 1), as the layers of a model need: e.g. per
+ * layer q/k/v (rows concatenated into one weight), o, gate/up
+ * (concatenated), down.  The attention, norms and activation between them
+ * are outside this library: every problem's x is an input of the call.  One persistent launch after the activation prep;
  * between problems a grid-wide barrier whose wait is bounded by the wall-
  * time limit (a wait that runs out sets the timeout bit of the device
  * status word, see tq_get_device_status, and the kernel returns).  The
