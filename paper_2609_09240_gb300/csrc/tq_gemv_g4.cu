@@ -616,9 +616,28 @@ __device__ __forceinline__ int unit_parts(int K, int SG, int split) {
 // stages, and all of this after the barrier, 1.61.  barrier_extra > 0 makes
 // every barrier wait for CTAs that do not exist, so that its bounded wait runs
 // out (the failure-path self-test).
+constexpr int kSeqP2 = 3;  // second-plane warps
+// Tiles of the second plane that these get through beside a stage of the
+// decode warps, about.
+constexpr int kSeqBeside = 16;
+// Whether problem P's second plane takes longer than its stages beside it, by
+// at least what it costs the decode warps to join in (about 2 us, as long as
+// 32 tiles of the second-plane warps): from 20 to 30 % salient groups on in
+// Qwen3-8B's problems.  Such a problem is dense: all warps share what exceeds
+// the tiles beside the stages, the decode warps theirs after their stages.
+// Six layers in order with 10, 30, 50 and 100 % salient groups: 195, 283, 320
+// and 382 us; by three warps alone 198, 300, 431 and 828; by the decode warps
+// before their stages, as this kernel once did, 276, 311, 344 and 426.
+// (The tiles are estimated, every group's last one half full; the warps that
+// share them count them.)
+__host__ __device__ inline bool dense_p2(const Problem &P, int stages, int ctas) {
+  return P.nnz > 0 && (P.nnz >> 4) + P.K / kGroup / 2 > kSeqBeside * ((stages > ctas ? stages : ctas) + 2 * ctas);
+}
+
 struct SeqWalk {
   const BatchParams *bp;
   int cta, ctas, p, unit, u_end, u, nst, tile, s, s_end;
+  bool dense;  // the decode warps take a part of the second plane
   __device__ void enter() {
     const Problem &P = bp->prob[p];
     const int G = P.K / kGroup, tiles = (P.N + kRows - 1) / kRows;
@@ -627,6 +646,7 @@ struct SeqWalk {
     const int split = share >= G ? 0 : share < 1 ? 1 : share;
     u = unit_parts(P.K, 8, split);
     nst = nstages(P.K, 8);
+    dense = dense_p2(P, tiles * nst, ctas);
     unit = share_at(tiles * u, cta, ctas);
     u_end = share_at(tiles * u, cta + 1, ctas);
     if (unit < u_end) locate();
@@ -659,9 +679,7 @@ __device__ __forceinline__ int ld_acquire(const int32_t *p) {
   return v;
 }
 
-constexpr int kSeqP2 = 3;  // second-plane warps
-
-// A second-plane warp's share of problem P's tiles (one token): the CTA's
+// A warp's share of problem P's second-plane tiles (one token): the CTA's
 // contiguous share of the index's 16-entry tiles, cut among the kSeqP2 warps,
 // in runs of tiles of one group (mm::p2_tiles with the group's activation
 // fragment of the per-group layout).  start() fetches what the first run
@@ -699,12 +717,20 @@ struct SeqP2 {
     }
     Cv = __ldg(reinterpret_cast<const float2 *>(P.wsCS + (int64_t)g * (mm::kCSGroup / 4)));
   }
-  __device__ __forceinline__ void start(const Problem &P, int cta, int ctas, int pw, int lane) {
+  // decode: the share of decode warp w (a dense problem), else of second-plane warp w
+  __device__ __forceinline__ void start(const Problem &P, int cta, int ctas, int w, int lane, bool decode,
+                                        bool any_dense) {
     t = end = n = 0;
     if (P.nnz <= 0) return;
     const int T2 = tiles_of(P);
-    const int lo = share_at(T2, cta, ctas), hi = share_at(T2, cta + 1, ctas);
-    t = lo + (hi - lo) * pw / kSeqP2, end = lo + (hi - lo) * (pw + 1) / kSeqP2;
+    int lo = share_at(T2, cta, ctas), hi = share_at(T2, cta + 1, ctas), warps = kSeqP2;
+    const int stages = (P.N + kRows - 1) / kRows * nstages(P.K, 8);
+    if (any_dense && dense_p2(P, stages, ctas)) {
+      const int rest = max(0, hi - lo - kSeqBeside * max(1, (stages + ctas - 1) / ctas));
+      const int mid = hi - rest + rest * kSeqP2 / (kSeqP2 + kWD1);
+      if (decode) lo = mid, warps = kWD1; else hi = mid;
+    }
+    t = lo + (hi - lo) * w / warps, end = lo + (hi - lo) * (w + 1) / warps;
     load_run(P, lane);
   }
   __device__ __forceinline__ void run(const Problem &P, int lane, uint32_t tag) {
@@ -732,7 +758,9 @@ __device__ __forceinline__ void prefetch_second_plane(const Problem &P, int cta,
 // ONE: a single problem, as a call of its own.  Such a call may share the GPU
 // with others, so its CTAs wait for none of each other: the last one to finish
 // (a ticket from the counter) stores all of y.
-template <bool F32, bool ONE>
+// DENSE: some problem is dense (dense_p2); without the decode warps' second
+// plane nothing spills.
+template <bool F32, bool ONE, bool DENSE>
 __global__ void __launch_bounds__((kWD1 + 1 + kSeqP2) * 32, 1)
     gemv_seq_kernel(const __grid_constant__ std::conditional_t<ONE, FewParams, BatchParams> params,
                     int32_t barrier_extra) {
@@ -795,6 +823,11 @@ __global__ void __launch_bounds__((kWD1 + 1 + kSeqP2) * 32, 1)
             }
         }
         if (++buf == (uint32_t)kNS) buf = 0, phase ^= 1u;
+      }
+      if (DENSE && ok && w.dense) {  // the decode warps' part of the second plane
+        SeqP2 sp;
+        sp.start(P, blockIdx.x, gridDim.x, warp, lane, true, true);
+        sp.run(P, lane, tag);
       }
       if constexpr (ONE) break;
       // the problem's barrier: every CTA's additions into y2 are done
@@ -889,7 +922,7 @@ __global__ void __launch_bounds__((kWD1 + 1 + kSeqP2) * 32, 1)
     bool stop = false;
     for (int p = 0; p < bp.count && !stop; ++p) {
       const Problem &P = bp.prob[p];
-      sp.start(P, blockIdx.x, gridDim.x, warp - WD - 1, lane);
+      sp.start(P, blockIdx.x, gridDim.x, warp - WD - 1, lane, false, DENSE);
       if (p > 0 && (stop = named_bar_any(2, kWorkers, *abort_ != 0))) break;
       if (warp == WD + 1 && lane == 0 && p + 1 < bp.count && bp.prob[p + 1].nnz > 0)
         prefetch_second_plane(bp.prob[p + 1], blockIdx.x, gridDim.x);
@@ -1165,13 +1198,20 @@ cudaError_t launch_gemv_seq(const BatchParams &bp, int num_sms, int barrier_extr
   if (bp.M != 1 || bp.count < 1 || (one && bp.count != 1)) return cudaErrorInvalidValue;
   const int ctas = std::min(num_sms, 256);
   constexpr int threads = (g4::kWD1 + 1 + g4::kSeqP2) * 32;
-  if (!one)
-    return launch_big_smem(bp.out_f32 ? g4::gemv_seq_kernel<true, false> : g4::gemv_seq_kernel<false, false>, ctas, threads,
-                           g4::kDynBytes, s, bp, (int32_t)barrier_extra);
-  FewParams few;
-  copy_params(few, bp);
-  return launch_big_smem(bp.out_f32 ? g4::gemv_seq_kernel<true, true> : g4::gemv_seq_kernel<false, true>, ctas, threads,
-                         g4::kDynBytes, s, few, (int32_t)barrier_extra);
+  bool dense = false;
+  for (int i = 0; i < bp.count; ++i)
+    dense = dense || g4::dense_p2(bp.prob[i], g4::tiles_of(bp.prob[i]) * g4::nstages(bp.prob[i].K, 8), ctas);
+  const auto launch = [&](auto dense_c) {
+    constexpr bool D = decltype(dense_c)::value;
+    if (!one)
+      return launch_big_smem(bp.out_f32 ? g4::gemv_seq_kernel<true, false, D> : g4::gemv_seq_kernel<false, false, D>, ctas,
+                             threads, g4::kDynBytes, s, bp, (int32_t)barrier_extra);
+    FewParams few;
+    copy_params(few, bp);
+    return launch_big_smem(bp.out_f32 ? g4::gemv_seq_kernel<true, true, D> : g4::gemv_seq_kernel<false, true, D>, ctas,
+                           threads, g4::kDynBytes, s, few, (int32_t)barrier_extra);
+  };
+  return dense ? launch(std::true_type{}) : launch(std::false_type{});
 }
 
 }  // namespace tq

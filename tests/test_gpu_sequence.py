@@ -86,3 +86,38 @@ def test_sequence_matches_batched(H):
     for (_, _, yb), (_, _, ys), (y_ref, a_ref) in zip(items_b, items_s, refs):
         H.assert_close(yb.float().cpu().numpy(), y_ref, a_ref)
         H.assert_close(ys.float().cpu().numpy(), y_ref, a_ref)
+
+
+def _mixed(H, problems):
+    """(N, K, salient share) in order and each alone, against the oracle on
+    sampled rows."""
+    from paper_2609_09240_gb300 import tq
+    items, refs = [], []
+    for i, (N, K, frac) in enumerate(problems):
+        w = wl.gen_weights(N, K, frac, config=12, proj=i)
+        xb = wl.gen_x(1, K, config=12, proj=i)
+        rows = np.sort(np.random.default_rng(N + i).choice(N, size=min(N, 400), replace=False)).astype(np.int32)
+        refs.append((rows,) + H.oracle_ref(w, xb, rows=rows))
+        items.append((H.pack_on_gpu(w), H.dev(xb), torch.empty((1, N), dtype=torch.float16, device="cuda")))
+
+    def check():
+        H.device_status_ok()
+        for (_, _, y), (rows, y_ref, a_ref) in zip(items, refs):
+            H.assert_close(y.float().cpu().numpy().astype(np.float64)[:, rows], y_ref, a_ref)
+
+    batch = tq.Batch(1, items)
+    for run in (lambda: tq.tq_linear_sequence(batch), lambda: [tq.tq_linear(x, w, y=y) for w, x, y in items]):
+        for _ in range(2):
+            for _, _, y in items:
+                y.fill_(float("nan"))
+            run()
+            check()
+
+
+@pytest.mark.parametrize("problems", [
+    [(40_001, 512, 1.0), (600, 1024, 0.2), (8000, 2048, 1.0), (300, 640, 0.0), (8000, 2048, 0.95)],  # dense ones among others
+    [(29_176, 512, 1.0), (29_180, 512, 1.0)],  # the last that the second-plane warps take alone, the first shared one
+    [(1000, 16_384, 1.0), (129, 65_536, 1.0), (70_000, 256, 1.0)],
+])
+def test_dense_second_planes(H, problems):
+    _mixed(H, problems)
