@@ -1531,18 +1531,24 @@ static cudaError_t launch_sequence(const BatchParams &bp_in, int barrier_extra, 
 
 // One token, one weight with an indexed second plane: both planes in one
 // kernel (the dependency-ordered one's variant for a single problem), instead
-// of one after the other in two.  10 % salient, as calls in a row: 2560 x 4096
-// 13.2 us against 17.6, 12288 x 4096 16.9 against 23.7, 49152 x 4096 33.8
-// against 42.5; 151936 x 4096 84 against 97, but 167 against 163 with 30 %
-// salient (its three second-plane warps then bind), so larger weights keep the
-// two kernels.  Without a second plane the first plane's kernel alone is as
-// fast (1024 x 2560: 11.1 against 12.3).
+// of one after the other in two.  It saves about 5 us of launches, and the
+// second plane's time (1 us for about 15000 salient groups), which runs beside
+// the first; it loses 0.7 us with each stage of its busiest CTA, which has
+// whole tiles from a tile per CTA up.  10 % salient, as calls in a row: 2560 x
+// 4096 13.2 us against 17.6, 12288 x 4096 16.9 against 23.7, 49152 x 4096 33.9
+// against 40.4, 151936 x 4096 82.9 against 92.0; with 50 % 68 and 85, 44 and 85,
+// 112 and 226 for the last three (dense second planes: tq_gemv_g4.cu), but with
+// 1 % 33.4 and 31.7 for 49152 x 4096 and 68 and 62 for 151936 x 4096, which
+// keep the two kernels.  Without a second plane the first plane's kernel alone
+// is as fast (1024 x 2560: 11.1 against 12.3).
 static bool one_launch(const BatchParams &bp) {
   if (!g4::takes(bp) || bp.M != 1 || bp.count != 1) return false;
   const Problem &P = bp.prob[0];
   if (P.nnz <= 0 || !P.p2idx) return false;
-  const int64_t units = (int64_t)((P.N + g4::kRows - 1) / g4::kRows) * g4::nstages(P.K, 8);
-  return units <= 16 * (int64_t)num_sms_mm();
+  const int64_t sms = num_sms_mm(), tiles = (P.N + g4::kRows - 1) / g4::kRows, nst = g4::nstages(P.K, 8);
+  if (tiles * nst > 16 * sms) return false;
+  const int64_t busiest = tiles >= sms ? (tiles + sms - 1) / sms * nst : (tiles * nst + sms - 1) / sms;
+  return P.nnz >= 15000 * (busiest - 5);
 }
 
 template <bool F32>

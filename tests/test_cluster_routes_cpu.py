@@ -1,4 +1,4 @@
-"""Which kernels a call launches on a GPU that holds fewer thread-block
+"""Which kernels a call launches, also on a GPU that holds fewer thread-block
 clusters, or none, or cannot say: the CUDA runtime is replaced by a fake that
 records launches (nothing runs), so no GPU is needed."""
 import json
@@ -64,17 +64,17 @@ p = lambda i: ctypes.c_void_p(0x10000 * (i + 1))  # never dereferenced
 def ternarize(N, K, nnz):
     return L.tq_ternarize(N, K, p(0), nnz, 4, p(1), p(2), p(3), p(4), p(5), p(6), p(7), p(8), 1 << 40, p(9), None)
 
-def prefill(M, N, K):
+def prefill(M, N, K, nnz=0):
     w = tq.tq_weight()
-    w.N, w.K, w.group, w.nnz = N, K, 128, 0
-    w.plane1 = w.salience = w.rowptr = w.scale1 = w.offset = 0x10000
+    w.N, w.K, w.group, w.nnz = N, K, 128, nnz
+    w.plane1 = w.salience = w.rowptr = w.scale1 = w.offset = w.plane2 = w.scale2 = w.p2index = 0x10000
     return L.tq_linear(M, N, K, ctypes.byref(w), p(0), p(1), p(2), 1 << 40, None)
 
 out = []
 for dev, clusters, call in json.loads(sys.argv[2]):
     F.fake_clusters(dev, clusters)
     F.fake_reset(dev)
-    rc = {"ternarize": ternarize, "prefill": prefill}[call[0]](*call[1:])
+    rc = {"ternarize": ternarize, "prefill": prefill, "linear": prefill}[call[0]](*call[1:])
     log = (ctypes.c_int * 256)()
     n = F.fake_log(log)
     out.append([rc, list(log[:n]), F.fake_last()])
@@ -125,3 +125,17 @@ def test_ternarize_selects_without_a_cluster(launches):
     assert no == [0, [1] * 9, 0] and failed == [0, [1] * 9, 0]
     too_many = ("ternarize", 26609, 128, 200)  # keys beyond the cluster's shared memory
     assert launches((0, 1, too_many)) == [[0, [1] * 9, 0]]
+
+
+def test_one_token_planes_in_one_kernel(launches):
+    """Prep and one kernel for both planes, or prep, second plane, first plane:
+    few salient groups in many stages take the two kernels."""
+    salient = lambda N, K, share: int(N * (K // 128) * share)
+    cases = [((1, 2560, 4096, 1), 2), ((1, 4096, 12288, salient(4096, 12288, 1.0)), 2),
+             ((1, 49152, 4096, salient(49152, 4096, 0.1)), 2), ((1, 49152, 4096, salient(49152, 4096, 0.01)), 3),
+             ((1, 151936, 4096, salient(151936, 4096, 0.3)), 2), ((1, 151936, 4096, salient(151936, 4096, 0.01)), 3),
+             ((1, 40000, 8192, 15000 * 11), 2), ((1, 40000, 8192, 15000 * 11 - 1), 3),  # 16 stages on the busiest SM
+             ((1, 200000, 4096, salient(200000, 4096, 0.3)), 3),  # more than 16 on every SM
+             ((1, 2560, 4096, 0), 2)]  # no second plane
+    got = launches(*[(0, 0, ("linear", *args)) for args, _ in cases])
+    assert got == [[0, [1] * n, 0] for _, n in cases]
