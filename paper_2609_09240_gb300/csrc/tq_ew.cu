@@ -44,7 +44,7 @@ struct Prob {
   const int32_t *idx_off;      // correction index (or null): offsets [N nb + 1]
   const uint16_t *idx;         //   and entries
   const __half *x;             // [M][K]
-  const float *ydense;         // [M][N]
+  float *ydense;               // [M][N]
   void *y;                     // [M][N], fp16 or fp32
   int32_t N, K, S, blocks;     // blocks = 0: the problem is the other kernel's
   int64_t w_begin;             // N G of the index kernel's problems before it
@@ -333,6 +333,35 @@ __device__ __forceinline__ void staged_acts(uint32_t a, float (&x)[MT]) {
   }
 }
 
+// Adds those of the index's first and last entries that are read alone
+// (tq_ew_pairs.cuh) and lie in rows [r_lo, r_hi) to the plane-1 result y [N] of
+// the token whose activations x are (the warp that has the rows, before it
+// reads their y).
+__device__ __forceinline__ void add_alone(const Prob &w, const unsigned short *x, float *y, int r_lo, int r_hi) {
+  const int nb = (w.K + kIdxBlock - 1) / kIdxBlock, odd = (int)(((uintptr_t)w.idx >> 1) & 1u);
+  const int entries = __ldg(w.idx_off + (int64_t)w.N * nb);
+#pragma unroll 1
+  for (int side = 0; side < 2; ++side) {
+    const int i = side ? entries - 1 : 0;
+    const int64_t lo = (int64_t)r_lo * nb, hi = (int64_t)r_hi * nb;
+    if (!read_alone(side, odd, entries) || i < __ldg(w.idx_off + lo) || i >= __ldg(w.idx_off + hi)) continue;
+    int64_t f = lo, end = hi;  // the entry's block: the last that begins at or before it
+    while (end - f > 1) {
+      const int64_t mid = (f + end) / 2;
+      if (__ldg(w.idx_off + mid) <= i) f = mid; else end = mid;
+    }
+    const int n = (int)(f / nb), b = (int)(f - (int64_t)n * nb);
+    const int en = __ldg(w.idx + i), code = en >> kIdxShift, q = code / 9;
+    if (code >= 27) continue;
+    const __half *mu = w.mu + (int64_t)n * 4, *a0 = w.a0 + (int64_t)n * 4;
+    float wt = (__half2float(mu[q]) - __half2float(mu[3])) +
+               (__half2float(a0[q]) - __half2float(a0[3])) * (float)(code / 3 % 3 - 1);
+    if (q < 2) wt += __half2float(w.a1[(int64_t)n * 2 + q]) * (float)(code % 3 - 1);
+    const int k = min(b * kIdxBlock + (en & (kIdxBlock - 1)), w.K - 1);
+    y[n] = fmaf(wt, __half2float(__ushort_as_half(__ldg(x + k))), y[n]);
+  }
+}
+
 // The same correction from the correction index.  An entry names its element
 // k (within its block of 2048) and code = 9 q + 3 d0 + d1 (digits d = trit +
 // 1), whose weight (mu_q - mu_3) + (alpha0_q - alpha0_3) T0 + alpha1_q T1 is
@@ -393,6 +422,14 @@ __global__ void __launch_bounds__(kIdxThreads, MT == 8 || (!STAGED && MT > 2) ? 
     if (b_lo >= b_hi) continue;
     const unsigned short *xm = reinterpret_cast<const unsigned short *>(w.x) + (int64_t)m0 * K;
     const int nb = (K + kIdxBlock - 1) / kIdxBlock;
+    // the warp's rows, their first and last offsets and the index's last one, on
+    // the way while x is staged (waited for after it, the last one, which every
+    // warp reads, cost a Qwen3-8B layer 1.2 us)
+    const int r_lo = b_lo + (b_hi - b_lo) * warp / kIdxWarps, r_hi = b_lo + (b_hi - b_lo) * (warp + 1) / kIdxWarps;
+    const int blocks = (r_hi - r_lo) * nb;
+    const int32_t *offs = w.idx_off + (int64_t)r_lo * nb;
+    const int entries = __ldg(w.idx_off + (int64_t)N * nb), o0 = __ldg(offs), o1 = __ldg(offs + min(1, blocks)),
+              o2 = __ldg(offs + min(2, blocks)), oN = __ldg(offs + blocks);
     if (STAGED) {
       __syncthreads();  // the warps are done with the problem before
       for (int i = threadIdx.x; i < nb * (kIdxBlock / 8); i += kIdxThreads) {
@@ -422,16 +459,12 @@ __global__ void __launch_bounds__(kIdxThreads, MT == 8 || (!STAGED && MT > 2) ? 
       __syncthreads();
     }
     grid_dep_wait();  // the plane-1 pass (returns at once from the second time on)
-    const int r_lo = b_lo + (b_hi - b_lo) * warp / kIdxWarps, r_hi = b_lo + (b_hi - b_lo) * (warp + 1) / kIdxWarps;
     if (r_lo >= r_hi) continue;
     // entries as aligned pairs, but for the index's first and last where a word
-    // of theirs reaches beyond it (tq_ew_pairs.cuh): their rows add them alone
+    // of theirs reaches beyond it (tq_ew_pairs.cuh): these go into ydense
     const int odd = (int)(((uintptr_t)w.idx >> 1) & 1u);
     const uint32_t *iw = reinterpret_cast<const uint32_t *>(w.idx - odd);
-    const int32_t *offs = w.idx_off + (int64_t)r_lo * nb;
-    const int blocks = (r_hi - r_lo) * nb, entries = __ldg(w.idx_off + (int64_t)N * nb), last = pairs_end(odd, entries);
-    const bool alone = (read_alone(false, odd, entries) && __ldg(offs) == 0) ||
-                       (read_alone(true, odd, entries) && __ldg(offs + blocks) == entries);
+    const int last = pairs_end(odd, entries);
     auto off_at = [&](int i) { return pairs_clamp(__ldg(offs + i), odd, last); };
     auto load_pairs = [&](uint32_t (&v)[kIdxAhead], int e, int e1) {
       const int first = (e + odd) >> 1, c = ((e1 + odd + 1) >> 1) - first;
@@ -450,10 +483,12 @@ __global__ void __launch_bounds__(kIdxThreads, MT == 8 || (!STAGED && MT > 2) ? 
     };
     auto h2f = [](unsigned short v) { return __half2float(__ushort_as_half(v)); };
     load_params(r_lo);
-    int e = off_at(0), e1 = off_at(1);
-    int e2 = blocks > 1 ? off_at(2) : e1;  // the next block's end
+    int e = pairs_clamp(o0, odd, last), e1 = pairs_clamp(o1, odd, last);
+    int e2 = pairs_clamp(o2, odd, last);  // the next block's end
     uint32_t v[kIdxAhead];
     load_pairs(v, e, e1);
+    if ((o0 == 0 && read_alone(false, odd, entries)) || (oN == entries && read_alone(true, odd, entries)))
+      if (lane < mt && lane < MT) add_alone(w, xm + (int64_t)lane * K, w.ydense + (int64_t)(m0 + lane) * N, r_lo, r_hi);
     int f = 0;  // the block among the run's
     for (int n = r_lo; n < r_hi; ++n) {
       float a = (h2f(h[0]) - h2f(h[1])) + (h2f(h[2]) - h2f(h[3])) * (float)(d0 - 1);
@@ -508,10 +543,20 @@ __global__ void __launch_bounds__(kIdxThreads, MT == 8 || (!STAGED && MT > 2) ? 
           }
         }
         if constexpr (STAGED) {
-          for (int i = 2 * (lane + 32 * kIdxAhead); i < c; i += 64) {
+          const int i0t = 2 * (lane + 32 * kIdxAhead);
+          auto tail = [&](int i) {
             const uint32_t r = __ldg(iw + ((e + odd) >> 1) + (i >> 1));
             add(r, true);
             add(r >> 16, i + 1 < c);
+          };
+          // (two steps at once for four and eight tokens: the compiler's own
+          // choice, faster for one and two, is 15 % slower for four with every
+          // element indexed)
+          if constexpr (MT >= 4) {
+#pragma unroll 2
+            for (int i = i0t; i < c; i += 64) tail(i);
+          } else {
+            for (int i = i0t; i < c; i += 64) tail(i);
           }
         } else {  // as many gathers under way as for the first entries
           for (int i1 = i0 + 64 * kIdxAhead; i1 - i0 < c; i1 += 64 * kIdxAhead) {
@@ -529,16 +574,6 @@ __global__ void __launch_bounds__(kIdxThreads, MT == 8 || (!STAGED && MT > 2) ? 
         e = e1, e1 = e2, e2 = e3;
 #pragma unroll
         for (int j = 0; j < kIdxAhead; ++j) v[j] = u[j];
-      }
-      if (alone) {
-        const int32_t *ro = offs + (int64_t)(n - r_lo) * nb;
-        for (int side = 0; side < 2; ++side) {
-          const int i = side ? entries - 1 : 0;
-          if (!read_alone(side, odd, entries) || i < __ldg(ro) || i >= __ldg(ro + nb)) continue;
-          int b = 0;  // the entry's block
-          while (__ldg(ro + b + 1) <= i) ++b;
-          add_at(__ldg(w.idx + i), lane == 0, b);
-        }
       }
       float mine = 0.f;
 #pragma unroll

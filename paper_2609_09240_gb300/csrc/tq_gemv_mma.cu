@@ -1535,10 +1535,10 @@ static cudaError_t launch_sequence(const BatchParams &bp_in, int barrier_extra, 
 // second plane's time (1 us for about 15000 salient groups), which runs beside
 // the first; it loses 0.7 us with each stage of its busiest CTA, which has
 // whole tiles from a tile per CTA up.  10 % salient, as calls in a row: 2560 x
-// 4096 13.2 us against 17.6, 12288 x 4096 16.9 against 23.7, 49152 x 4096 33.9
-// against 40.4, 151936 x 4096 82.9 against 92.0; with 50 % 68 and 85, 44 and 85,
-// 112 and 226 for the last three (dense second planes: tq_gemv_g4.cu), but with
-// 1 % 33.4 and 31.7 for 49152 x 4096 and 68 and 62 for 151936 x 4096, which
+// 4096 12.8 us against 16.9, 12288 x 4096 16.2 against 21.4, 49152 x 4096 34.0
+// against 40.3, 151936 x 4096 83.0 against 91.8; with 50 % the last three take
+// 20, 43 and 123 against 34, 86 and 226 (dense second planes: tq_gemv_g4.cu),
+// but with 1 % 33.5 and 68.4 against 31.7 and 62.7 for the last two, which then
 // keep the two kernels.  Without a second plane the first plane's kernel alone
 // is as fast (1024 x 2560: 11.1 against 12.3).
 static bool one_launch(const BatchParams &bp) {

@@ -184,7 +184,7 @@ def _p(t):
 
 def _stream(stream):
     if stream is None:
-        # the current stream's handle without a Stream object around it (0.4 us
+        # the current stream's handle without a Stream object around it (0.3 us
         # a call instead of 3.0; every caller's tensors have initialized CUDA);
         # a torch without these private functions gives the object
         try:
