@@ -984,7 +984,7 @@ __global__ void __launch_bounds__(c_threads(TWO), 1)
   // after it); the main kernel may start its set-up meanwhile
   grid_dep_wait();
   grid_dep_launch_next();
-  const int MB = ONE ? 1 : bp.M, g16 = lane >> 2, c = lane & 3, quad = lane & ~3;
+  const int MB = ONE ? 1 : bp.M, g16 = lane >> 2, c = lane & 3;
   const uint32_t tag = kLutShared | ((uint32_t)lane << 2);
   const int count = cb.count, total = cb.base[count];
   for (;;) {

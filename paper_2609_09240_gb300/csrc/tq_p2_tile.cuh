@@ -119,59 +119,59 @@ __device__ __forceinline__ void p2_tiles(const Problem &P, int MB, int GL, const
                                          uint2 (&pre)[kCDepth][2], const uint32_t *b, const uint32_t *b2, float2 Cv,
                                          float2 Cv2, int lane, uint32_t tag) {
   const int c = lane & 3, quad = lane & ~3;
-    // lane c's window words jw and jw + 4 are slot words 2 jw, 2 jw + 1; the row is the second
-    // word of the lane with jw = 3, s2 a half of the first word of jw = 0 (record at byte 2)
-    // or of the second word of jw = 2 (record at byte 0)
-    const int ws = win_start(GL), odd = GL & 1;
-    const int c_row = quad + ((3 + ws) & 3), c_s2 = quad + (((odd ? 0 : 2) + ws) & 3);
-    float *y2 = P.y2();
-    for (int t = 0; t < n; t += kCDepth) {
+  // lane c's window words jw and jw + 4 are slot words 2 jw, 2 jw + 1; the row is the second
+  // word of the lane with jw = 3, s2 a half of the first word of jw = 0 (record at byte 2)
+  // or of the second word of jw = 2 (record at byte 0)
+  const int ws = win_start(GL), odd = GL & 1;
+  const int c_row = quad + ((3 + ws) & 3), c_s2 = quad + (((odd ? 0 : 2) + ws) & 3);
+  float *y2 = P.y2();
+  for (int t = 0; t < n; t += kCDepth) {
 #pragma unroll
-      for (int k = 0; k < kCDepth; ++k) {
-        if (t + k < n) {
-          const uint2 r0 = pre[k][0], r1 = pre[k][1];
-          if (t + k + kCDepth < n) {
-            const unsigned char *p = src + (int64_t)(t + k + kCDepth) * 512;
-            pre[k][0] = __ldg(reinterpret_cast<const uint2 *>(p));
-            pre[k][1] = __ldg(reinterpret_cast<const uint2 *>(p + 256));
+    for (int k = 0; k < kCDepth; ++k) {
+      if (t + k < n) {
+        const uint2 r0 = pre[k][0], r1 = pre[k][1];
+        if (t + k + kCDepth < n) {
+          const unsigned char *p = src + (int64_t)(t + k + kCDepth) * 512;
+          pre[k][0] = __ldg(reinterpret_cast<const uint2 *>(p));
+          pre[k][1] = __ldg(reinterpret_cast<const uint2 *>(p + 256));
+        }
+        uint32_t aL[20], aH[20];
+        decode_words(r0.x, r0.y, tag, aL);
+        decode_words(r1.x, r1.y, tag, aH);
+        float d[4], d2[4] = {0.f, 0.f, 0.f, 0.f};
+        group_mma(aL, aH, b, d);
+        if (TWO) group_mma(aL, aH, b2, d2);
+        const uint32_t sw0 = __shfl_sync(0xffffffffu, odd ? r0.x : r0.y, c_s2);
+        const uint32_t sw1 = __shfl_sync(0xffffffffu, odd ? r1.x : r1.y, c_s2);
+        const float s2v0 = odd ? half_of<false>(sw0) : half_of<true>(sw0);
+        const float s2v1 = odd ? half_of<false>(sw1) : half_of<true>(sw1);
+        if (ONE) {
+          // every column of D is token 0: the lane holding the rows adds
+          if (lane == c_row) {
+            const int n0 = (int)r0.y, n1 = (int)r1.y;
+            if (n0 >= 0 && n0 < P.N) atomicAdd(&y2[n0], s2v0 * (d[0] - Cv.x));
+            if (n1 >= 0 && n1 < P.N) atomicAdd(&y2[n1], s2v1 * (d[2] - Cv.x));
           }
-          uint32_t aL[20], aH[20];
-          decode_words(r0.x, r0.y, tag, aL);
-          decode_words(r1.x, r1.y, tag, aH);
-          float d[4], d2[4] = {0.f, 0.f, 0.f, 0.f};
-          group_mma(aL, aH, b, d);
-          if (TWO) group_mma(aL, aH, b2, d2);
-          const uint32_t sw0 = __shfl_sync(0xffffffffu, odd ? r0.x : r0.y, c_s2);
-          const uint32_t sw1 = __shfl_sync(0xffffffffu, odd ? r1.x : r1.y, c_s2);
-          const float s2v0 = odd ? half_of<false>(sw0) : half_of<true>(sw0);
-          const float s2v1 = odd ? half_of<false>(sw1) : half_of<true>(sw1);
-          if (ONE) {
-            // every column of D is token 0: the lane holding the rows adds
-            if (lane == c_row) {
-              const int n0 = (int)r0.y, n1 = (int)r1.y;
-              if (n0 >= 0 && n0 < P.N) atomicAdd(&y2[n0], s2v0 * (d[0] - Cv.x));
-              if (n1 >= 0 && n1 < P.N) atomicAdd(&y2[n1], s2v1 * (d[2] - Cv.x));
-            }
-          } else {
-            const int rows[2] = {__shfl_sync(0xffffffffu, (int)r0.y, c_row),
-                                 __shfl_sync(0xffffffffu, (int)r1.y, c_row)};
-            const float s2v[2] = {s2v0, s2v1};
+        } else {
+          const int rows[2] = {__shfl_sync(0xffffffffu, (int)r0.y, c_row),
+                               __shfl_sync(0xffffffffu, (int)r1.y, c_row)};
+          const float s2v[2] = {s2v0, s2v1};
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-              const int nr = rows[h];
-              if (nr < 0 || nr >= P.N) continue;
+          for (int h = 0; h < 2; ++h) {
+            const int nr = rows[h];
+            if (nr < 0 || nr >= P.N) continue;
 #pragma unroll
-              for (int ii = 0; ii < 2; ++ii) {
-                const int m = 2 * c + ii;
-                if (m < MB) atomicAdd(&y2[(int64_t)nr * MB + m], s2v[h] * (d[2 * h + ii] - (ii ? Cv.y : Cv.x)));
-                if (TWO && 8 + m < MB)
-                  atomicAdd(&y2[(int64_t)nr * MB + 8 + m], s2v[h] * (d2[2 * h + ii] - (ii ? Cv2.y : Cv2.x)));
-              }
+            for (int ii = 0; ii < 2; ++ii) {
+              const int m = 2 * c + ii;
+              if (m < MB) atomicAdd(&y2[(int64_t)nr * MB + m], s2v[h] * (d[2 * h + ii] - (ii ? Cv.y : Cv.x)));
+              if (TWO && 8 + m < MB)
+                atomicAdd(&y2[(int64_t)nr * MB + 8 + m], s2v[h] * (d2[2 * h + ii] - (ii ? Cv2.y : Cv2.x)));
             }
           }
         }
       }
     }
+  }
 }
 
 }  // namespace mm

@@ -212,9 +212,6 @@ struct Bars2 {
 };
 static_assert(sizeof(Bars2) <= 256, "prefill2 barriers");
 
-__device__ __forceinline__ void cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
 // a float into another cluster CTA's shared memory, at this CTA's address a
 __device__ __forceinline__ void st_remote(uint32_t a, int rank, float v) {
   asm volatile("{\n.reg .b32 r;\nmapa.shared::cluster.u32 r, %0, %1;\nst.shared::cluster.f32 [r], %2;\n}" ::"r"(a),

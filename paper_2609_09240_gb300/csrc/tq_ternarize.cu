@@ -408,9 +408,6 @@ __host__ __device__ inline int64_t select_keys(int N, int SW) {
   return (int64_t)((N + kSelCtas - 1) / kSelCtas) * SW * 32;  // per CTA, rows padded to whole words
 }
 
-__device__ __forceinline__ void cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
 // The 32-bit word at shared address `addr` of CTA `rank` of the cluster.
 __device__ __forceinline__ uint32_t ld_cluster(const uint32_t *p, int rank) {
   uint32_t a, v;
