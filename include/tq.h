@@ -436,8 +436,10 @@ TQ_API size_t tq_ew_workspace_bytes(int32_t M, int32_t N, int32_t K);
 /* y = x W-hat^T for the element-wise form, x fp16 [M][K] (16-byte aligned),
  * y fp16 [M][N] (tq_ew_linear_f32out: fp32).  Plane 1 with mask 3's
  * parameters runs through tq_linear's kernels; a second kernel adds, per
- * row, the elements of masks 0..2 and writes y.  The fp32 sums are added in
- * a fixed order. */
+ * row, the elements of masks 0..2 and writes y.  That kernel's fp32 sums are
+ * added in a fixed order; with one or two tokens plane 1's are not where
+ * several SMs share a tile of rows, so results may then differ in the last
+ * bits from run to run. */
 TQ_API tq_status tq_ew_linear(int32_t M, int32_t N, int32_t K, const tq_ew_weight *w, const uint16_t *x, uint16_t *y,
                               void *workspace, size_t workspace_bytes, void *stream);
 TQ_API tq_status tq_ew_linear_f32out(int32_t M, int32_t N, int32_t K, const tq_ew_weight *w, const uint16_t *x,
