@@ -511,11 +511,11 @@ def run_ternarize(args, ws, rank, local):
         "roofline": {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "Top/s",
                      "frac": achieved / peak, "traffic": None,
                      "peak_kind": f"{FP32_LANES_PER_SM} fp32 lanes x {sms} SMs x {mhz:.0f} MHz (derived, not measured)",
-                     "kernel": "whole tq_ternarize call (nine launches per projection, 63 per step)",
+                     "kernel": "whole tq_ternarize call (three launches per projection, 21 per step)",
                      "ops_per_step": ops},
         "e2e": {"value": n_weights / (e2e_ms * 1e-3) / 1e9, "unit": "Gweights/s", "h2d_bytes_per_step": h2d,
                 "d2h_bytes_per_step": d2h},
-        "gpu_launches": 9 * 7 * steps,
+        "gpu_launches": 3 * 7 * steps,
         "clocks": clocks,
     }
     if rank == 0 and not args.no_cpu_baseline:
@@ -708,7 +708,7 @@ def sub_unbatched_8b(items, dev, batched_ms):
     return {"workload": "qwen3-8b step, each projection its own tq_linear call, M=1",
             "us_per_layer": ms * 1e3 / layers, "us_per_layer_batched": batched_ms * 1e3 / layers,
             "ratio_to_batched": ms / batched_ms,
-            "timing": f"{len(items)} tq_linear calls (3 launches each) replayed as one CUDA graph"}
+            "timing": f"{len(items)} tq_linear calls (2 launches each) replayed as one CUDA graph"}
 
 
 def sub_prefill(dev, steps=20):

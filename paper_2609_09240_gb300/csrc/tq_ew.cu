@@ -382,8 +382,8 @@ __device__ __forceinline__ void add_alone(const Prob &w, const unsigned short *x
 // or activation address is one shift and one three-input AND-OR (tables and
 // blocks lie at multiples of their size), one token is staged as fp32, and
 // entries past a block's end are cut by predicates: 20
-// warp-instructions per 32 entries with all that surrounds them, 18.4 M for
-// one Qwen3-8B layer in 28.3 us (66 % of the issue slots; 54 MB, whose floor
+// warp-instructions per 32 entries with all that surrounds them, 19.4 M for
+// one Qwen3-8B layer in 27.8 us (66 % of the issue slots; 54 MB, whose floor
 // is 8 us), against 31.6 M in 39.5 us with one guarded entry per lane and
 // step, and 48 us with gathers from global memory.
 // STAGED = false reads x from global memory: K x tokens beyond a block's
