@@ -364,3 +364,24 @@ def test_linear_indexed_long_rows(H, M, N, K, cover):
     y = tq.tq_ew_linear(H.dev(xb), _indexed(H, w), f32=True)
     H.device_status_ok()
     H.assert_close(y.cpu().numpy().astype(np.float64), y_ref, a_ref)
+
+
+@pytest.mark.parametrize("count", [8, 9, 40])
+@pytest.mark.parametrize("M", [1, 5])
+def test_batched_parameter_sizes(H, count, M):
+    """The most problems that fit the small launch parameters, one more, and
+    many: indexed, plain and empty ones."""
+    from paper_2609_09240_gb300 import tq
+    items, refs = [], []
+    for i in range(count):
+        N, K = 20 + 13 * (i % 7), 128 * (1 + 5 * (i % 4))
+        w = wl.gen_ew_weights(N, K, config=29, proj=i, coverage=(0.0, 0.0, 0.0) if i % 5 == 4 else (0.02, 0.05, 0.1))
+        xb = wl.gen_x(M, K, config=29, proj=i)
+        mp, p1, rp, p2, st = ew.pack(w.T0, w.T1, w.mask)
+        refs.append(ew.linear(xb, K, mp, p1, rp, p2, w.mu, w.a0, w.a1))
+        items.append((_pack(H, w) if i % 3 == 1 else _indexed(H, w), H.dev(xb),
+                      torch.full((M, N), float("nan"), dtype=torch.float16, device="cuda")))
+    tq.tq_ew_linear_batched(tq.EwBatch(M, items))
+    H.device_status_ok()
+    for (_, _, y), (y_ref, a_ref) in zip(items, refs):
+        H.assert_close(y.float().cpu().numpy().astype(np.float64), y_ref, a_ref)
