@@ -411,6 +411,8 @@ def alu_peak_tops(dev, sm_max_mhz=None):
     The SM count is the device's own; the clock is the maximum that the clock
     sampler read during the run, else 2070 MHz (the part's maximum SM clock).
     """
+    import torch
+
     sms = torch.cuda.get_device_properties(dev).multi_processor_count
     mhz = sm_max_mhz if sm_max_mhz else 2070.0
     return FP32_LANES_PER_SM * sms * mhz * 1e6 / 1e12, sms, mhz

@@ -55,3 +55,14 @@ def test_kernel_hash_ignores_comments(tmp_path, monkeypatch):
     assert bench.kernel_hash() == h0
     src.write_text(text.replace("kP2rTiles = 8;", "kP2rTiles = 9;", 1))
     assert "kP2rTiles = 9;" in src.read_text() and bench.kernel_hash() != h0
+
+
+def test_alu_peak_of_a_device(monkeypatch):
+    """128 fp32 lanes x SMs x clock, the SMs from the device's properties."""
+    import types
+
+    import bench
+    import torch
+    monkeypatch.setattr(torch.cuda, "get_device_properties", lambda dev: types.SimpleNamespace(multi_processor_count=152))
+    peak, sms, mhz = bench.alu_peak_tops(0, 2000.0)
+    assert sms == 152 and mhz == 2000.0 and peak == pytest.approx(128 * 152 * 2e9 / 1e12)
